@@ -149,14 +149,10 @@ bool make_geometry(int dim, int64_t N, Geometry* g) {
 }
 
 static int default_stencil(const qw_plan_s* p) {
-  // measured on GB300: BCC N = 512, the fused two-step kernel (one HBM pass per two steps,
-  // shared-memory bound) ahead of the one-step TMA kernel (HBM bound); the chain (N = 2^28),
-  // FUSED with four steps per launch ahead of PLAIN (232 against 209 G site-steps/s); the
-  // square lattice, PLAIN.  qw_plan_autotune re-measures on the device.
-  if (stencil_supported(p->g, p->dtype, QW_STENCIL_TMA2)) return QW_STENCIL_TMA2;
+  // measured on GB300: the chain (N = 2^28), FUSED with four steps per launch ahead of PLAIN (232
+  // against 209 G site-steps/s); the square lattice and BCC boxes of every size, PLAIN (BCC: the
+  // marching kernel, march3.cu).  qw_plan_autotune re-measures on the device.
   if (p->g.dim == 1 && fused_step_supported(p->g, p->dtype, p->fuse_depth, p->fuse_box)) return QW_STENCIL_FUSED;
-  if (stencil_supported(p->g, p->dtype, QW_STENCIL_TMA)) return QW_STENCIL_TMA;
-  if (stencil_supported(p->g, p->dtype, QW_STENCIL_VEC)) return QW_STENCIL_VEC;
   return QW_STENCIL_PLAIN;
 }
 
@@ -250,6 +246,7 @@ qw_status qw_plan_create(int dim, int64_t N, double mass, qw_dtype dtype, qw_pla
   p->elem_bytes = (dtype == QW_C64) ? 8 : 16;
   qw_status st = QW_OK;
   cudaError_t e = cudaGetDevice(&p->device);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&p->sms, cudaDevAttrMultiProcessorCount, p->device);
   if (e == cudaSuccess) e = cudaMalloc(&p->scratch, (size_t)g.elems * p->elem_bytes);
   if (e == cudaSuccess) e = cudaMalloc(&p->red_partials, sizeof(double) * 10 * kMom2MaxBlocks);
   if (e == cudaSuccess) e = cudaMalloc(&p->red_result, sizeof(double) * 16);
@@ -343,9 +340,16 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     QW_CHECK_CUDA(cudaMemsetAsync(p->scratch, kPoisonByte, (size_t)p->g.elems * p->elem_bytes, s));
   void* cur = psi;
   void* nxt = p->scratch;
+  int64_t march[5] = {0, 0, 0, 0, 0};  // PLAIN on BCC boxes: launches of 1..4 steps left
+  const bool marching = variant == QW_STENCIL_PLAIN && p->g.dim == 3;
+  if (marching) march3_schedule(p->g, p->dtype, nsteps, p->sms, march);
   for (int64_t i = 0; i < nsteps;) {
     int done = 1;
-    if (variant == QW_STENCIL_TMA2 && nsteps - i >= 2) {
+    if (marching) {
+      done = march[4] ? 4 : march[3] ? 3 : march[2] ? 2 : 1;
+      --march[done];
+      st = launch_march3(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, s);
+    } else if (variant == QW_STENCIL_TMA2 && nsteps - i >= 2) {
       st = launch_step_tma2(p->g, p->n, p->mass, cur, nxt, p->tma2_items, p->tma2_nitems, p->dev_flags,
                             p->dev_flags + 1, s);
       done = 2;

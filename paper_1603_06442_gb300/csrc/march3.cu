@@ -1,0 +1,167 @@
+// BCC boxes: several steps of the update rule per pass over HBM with the marching kernel of
+// qw_march.cuh (any M, complex64 and complex128), and the choice of its tile per box.
+//
+// complex64, one GB300, G site-steps/s of the kernel against the kernels it replaced (the two-step
+// TMA kernel for M % 64 = 0, one thread per site and step otherwise): M = 256: 214 against 121;
+// M = 125: 168 against 68; M = 64: 79 against 36.  It is bound by issue slots and dependent
+// latencies (2 warps per scheduler at ~250 registers; IPC 0.55, FP32 pipe 40%), no longer by
+// shared memory (40% of the wavefront peak) or HBM (31%), so what a tile recomputes in its halo
+// costs directly: the tile and the number of steps are chosen by the estimate below.
+// complex128: bound by the FP64 pipe (2 lanes a clock and SM): 48 FP64 instructions a site-step
+// instead of 104, one step a launch (every recomputed site costs): M = 64: 7.5 against 5.1.
+#include <cuda_runtime.h>
+
+#include "qw_march.cuh"
+
+namespace qw {
+namespace {
+
+// Instantiated tiles: KX cells per lane, KY rows per warp, T steps, NW warps, CTAs per SM; us per
+// half-layer of a CTA with the SM full (measured, which the estimate multiplies with the half-layers
+// of the longest CTA).
+struct Tile3 {
+  int kx, ky, t, nw, ctas;
+  double us;
+};
+template <typename R, int KX, int KY, int T, int NW, int CTAS>
+qw_status launch_tile(const March3<typename CplxOf<R>::T>& p, int grid, typename CoefOf<R>::T cf, cudaStream_t st) {
+  auto* k = march3d_kernel<R, KX, KY, T, NW, CTAS>;
+  constexpr int smem = march3_smem<R, KX, KY, NW>();
+  const qw_status s = smem_attr(k, smem);
+  if (s != QW_OK) return s;
+  k<<<grid, 32 * NW, smem, st>>>(p, cf);
+  QW_CHECK_LAUNCH("marching stencil launch");
+  return QW_OK;
+}
+
+#define QW_TILES3_C64(X)                                                                            \
+  X(1, 3, 4, 8, 1, 1.40) X(1, 2, 4, 8, 1, 1.05) X(1, 3, 3, 4, 2, 1.04) X(1, 4, 3, 4, 2, 1.42)       \
+  X(1, 4, 2, 4, 2, 1.25) X(1, 2, 1, 8, 2, 0.85)
+#define QW_TILES3_C128(X) X(2, 1, 1, 4, 2, 4.9) X(1, 1, 1, 8, 2, 5.0)
+
+const Tile3 kTiles64[] = {
+#define X(kx, ky, t, nw, ctas, us) {kx, ky, t, nw, ctas, us},
+    QW_TILES3_C64(X)};
+const Tile3 kTiles128[] = {QW_TILES3_C128(X)
+#undef X
+};
+
+template <typename C> March3<C> geometry3(const Geometry& g, const Tile3& s, int sms, int* grid) {
+  March3<C> p{};
+  const int M = (int)g.nx;
+  p.M = M;
+  p.perx = M <= 32 * s.kx && M % s.kx == 0;
+  p.lanes = p.perx ? M / s.kx : 32;
+  p.pery = s.nw * s.ky == M;
+  p.tx = p.perx ? M : 32 * s.kx - s.t;
+  p.ty = p.pery ? M : s.nw * s.ky - s.t;
+  p.ntx = (M + p.tx - 1) / p.tx;
+  p.nty = (M + p.ty - 1) / p.ty;
+  *grid = march3_split(p, s.t, sms * s.ctas);
+  return p;
+}
+
+double estimate3(const Geometry& g, const Tile3& s, int sms) {
+  int grid;
+  const March3<float2> p = geometry3<float2>(g, s, sms, &grid);
+  const int P = 2 * p.M;
+  int iters = p.rounds * (P + 2 * s.t);
+  if (p.rest) iters += (p.planes < P ? p.planes : P) + 2 * s.t;
+  return 4.0 + iters * s.us;  // us a launch: start and end, and the half-layers of the longest CTA
+}
+
+}  // namespace
+
+// us of a launch of `steps` steps (the best tile for it), or < 0 where no tile takes that many.
+double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
+  double best = -1.0;
+  const Tile3* t = dt == QW_C64 ? kTiles64 : kTiles128;
+  const int n = dt == QW_C64 ? (int)(sizeof(kTiles64) / sizeof(Tile3)) : (int)(sizeof(kTiles128) / sizeof(Tile3));
+  for (int i = 0; i < n; ++i)
+    if (t[i].t == steps) {
+      const double c = estimate3(g, t[i], sms);
+      if (best < 0 || c < best) best = c;
+    }
+  return best;
+}
+
+// Launches of 4, 3, 2 and 1 steps that make nsteps: the cheapest mix by the estimates above; an odd
+// number of launches ends in the scratch field and costs a copy of the field.
+void march3_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]) {
+  double cost[5];
+  for (int t = 1; t <= 4; ++t) cost[t] = march3_cost(g, dt, t, sms);
+  const double copy = 3.0 + 2.0 * (double)g.elems * (dt == QW_C64 ? 8 : 16) / 6.0e6;
+  double best = -1.0;
+  for (int64_t& c : count) c = 0;
+  // small counts of three of the sizes, the rest in launches of the fourth
+  for (int main = 1; main <= 4; ++main) {
+    if (cost[main] < 0) continue;
+    int64_t k[5] = {0, 0, 0, 0, 0};
+    const int a = main == 1 ? 2 : 1, b = main <= 2 ? 3 : 2, c = main <= 3 ? 4 : 3;
+    for (k[a] = 0; k[a] <= 4; ++k[a])
+      for (k[b] = 0; k[b] <= 4; ++k[b])
+        for (k[c] = 0; k[c] <= 4; ++k[c]) {
+          if ((k[a] && cost[a] < 0) || (k[b] && cost[b] < 0) || (k[c] && cost[c] < 0)) continue;
+          const int64_t left = nsteps - a * k[a] - b * k[b] - c * k[c];
+          if (left < 0 || left % main) continue;
+          k[main] = left / main;
+          const int64_t launches = k[1] + k[2] + k[3] + k[4];
+          double total = launches % 2 ? copy : 0.0;
+          for (int t = 1; t <= 4; ++t)
+            if (k[t]) total += (double)k[t] * cost[t];
+          if (best < 0 || total < best) {
+            best = total;
+            for (int t = 1; t <= 4; ++t) count[t] = k[t];
+          }
+        }
+  }
+}
+
+qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
+                        int sms, cudaStream_t st) {
+  const Tile3* t = dt == QW_C64 ? kTiles64 : kTiles128;
+  const int cnt = dt == QW_C64 ? (int)(sizeof(kTiles64) / sizeof(Tile3)) : (int)(sizeof(kTiles128) / sizeof(Tile3));
+  int best = -1;
+  double bc = 0.0;
+  for (int i = 0; i < cnt; ++i) {
+    if (t[i].t != steps) continue;
+    const double c = estimate3(g, t[i], sms);
+    if (best < 0 || c < bc) {
+      best = i;
+      bc = c;
+    }
+  }
+  if (best < 0) {
+    set_error("marching stencil: no kernel for %d steps", steps);
+    return QW_EINVAL;
+  }
+  int grid, i = 0;
+  auto planes = [&](auto& p) {
+    using C = std::remove_const_t<std::remove_pointer_t<std::remove_reference_t<decltype(p.out[0][0])>>>;
+    for (int c = 0; c < 2; ++c)
+      for (int q = 0; q < 4; ++q) {
+        p.in[c][q] = static_cast<const C*>(in) + (int64_t)(c * 4 + q) * g.vol;
+        p.out[c][q] = static_cast<C*>(out) + (int64_t)(c * 4 + q) * g.vol;
+      }
+  };
+  if (dt == QW_C64) {
+    March3<float2> p = geometry3<float2>(g, t[best], sms, &grid);
+    planes(p);
+    const Coef32 cf = make_coef32(3, n, m);
+#define X(kx, ky, T, nw, ctas, us) \
+  if (i++ == best) return launch_tile<float, kx, ky, T, nw, ctas>(p, grid, cf, st);
+    QW_TILES3_C64(X)
+  } else {
+    March3<double2> p = geometry3<double2>(g, t[best], sms, &grid);
+    planes(p);
+    const Coef64 cf = make_coef64(3, n, m);
+#undef X
+#define X(kx, ky, T, nw, ctas, us) \
+  if (i++ == best) return launch_tile<double, kx, ky, T, nw, ctas>(p, grid, cf, st);
+    QW_TILES3_C128(X)
+#undef X
+  }
+  return QW_EINVAL;
+}
+
+}  // namespace qw

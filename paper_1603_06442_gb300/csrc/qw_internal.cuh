@@ -119,6 +119,11 @@ qw_status launch_step_tma2(const Geometry& g, double n, double m, const void* in
                            int nitems, int* err, int* next_item, cudaStream_t st);
 qw_status launch_step_tma(const Geometry& g, double n, double m, const void* in, void* out, const int4* items,
                           int nitems, int* err, int* next_item, cudaStream_t st);
+// Marching kernels, BCC (march3.cu): `steps` updates out = U^steps in per launch, the steps between held
+// in registers.  march3_schedule: how many launches of 1..4 steps make nsteps.
+void march3_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]);
+qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
+                        int sms, cudaStream_t st);
 // FUSED: `steps` <= depth updates in one launch, box tiles of the field and a halo in shared
 // memory (complex64, any geometry whose tile fits shared memory; batch.cu).
 bool fused_step_supported(const Geometry& g, qw_dtype dt, int depth, const int* box);
@@ -240,6 +245,7 @@ struct qw_plan_s {
   double n;
   qw_dtype dtype;
   int device;
+  int sms;              // multiprocessors of the device
   size_t elem_bytes;
   int stencil;          // qw_stencil_variant in use (never AUTO after creation)
   int fuse_depth;       // FUSED variant: steps per launch and tile box (x, y, z cells)

@@ -89,6 +89,7 @@ template <typename C> __device__ __forceinline__ C csub(C a, C b) { return C{a.x
 template <typename C> __device__ __forceinline__ C rho(C z) { return C{z.x - z.y, z.x + z.y}; }
 template <typename C> __device__ __forceinline__ C rhob(C z) { return C{z.x + z.y, z.y - z.x}; }
 template <typename C> __device__ __forceinline__ C addi(C a, C b) { return C{a.x - b.y, a.y + b.x}; }  // a + i b
+template <typename C> __device__ __forceinline__ C subi(C a, C b) { return C{a.x + b.y, a.y - b.x}; }  // a - i b
 
 // square lattice, s = 4: the four outputs from the cells A = x-1, B = x+1, C = y-1, D = y+1
 // (sources of h = +e1, -e1, +e2, -e2) and the own cell.  From the tables above, rho = 1 + i:
@@ -136,51 +137,44 @@ __device__ __forceinline__ void site_update_2d(const typename CplxOf<R>::T* __re
 }
 
 // BCC, s = 4: output coset c at cell (x, y, z) reads coset 1-c at (per axis) m - 1 + c for
-// h = +1 and m + c for h = -1 (the site x - h of the other sublattice).  From the tables above,
-// with the sources s_{hx hy} of the plane of h_z = +1 and t_{hx hy} of the plane of h_z = -1,
-// components a, b, c, d, and rho = 1 + i:
-//   S0 = rhob [(a_{++} + b_{++}) + (a_{--} - b_{--})] + rho [(a_{+-} + b_{+-}) + (a_{-+} - b_{-+})]   (s)
-//   S1 = rho [(a_{++} + b_{++}) + (b_{--} - a_{--})] + rhob [(a_{+-} + b_{+-}) + (b_{-+} - a_{-+})]   (t)
-//   S2 = rhob (d_{--} - d_{++}) + rho (d_{-+} - d_{+-})  (s)  +  rho (c_{++} + c_{--}) + rhob (c_{+-} + c_{-+})  (t)
-//   S3 = rhob (d_{++} + d_{--}) + rho (d_{+-} + d_{-+})  (s)  +  rho (c_{--} - c_{++}) + rhob (c_{-+} - c_{+-})  (t)
-// (88 real additions instead of 128 term by term), then the mass step (finish).
+// h = +1 and m + c for h = -1 (the site x - h of the other sublattice).  The transition matrices are
+// products of one conditional shift per axis, so the sums factor axis by axis.  With sources
+// a, b, c, d and rho = 1 + i, rhob = 1 - i:
+//   upper spinor, per plane: X+- = a +- b at h_x = +-1; A = X+ + i X- of the row of h_y = +1,
+//     B = X+ - i X- of the row of h_y = -1; S0 = rhob (A + i B) of the plane of h_z = +1,
+//     S1 = rho (A - i B) of the plane of h_z = -1;
+//   lower spinor, per column: V = c + i d of the row of h_y = +1, W = c - i d of the row of
+//     h_y = -1, with c of the plane of h_z = -1 and d of the plane of h_z = +1;
+//     G = rho (V - i W) of the column of h_x = +1, H = rhob (V + i W) of the column of h_x = -1;
+//     S2 = H + G, S3 = H - G
+// (52 real additions for a site on its own, 32 where neighbours share X, A, B, V, W, G, H as in
+// qw_march.cuh, instead of 128 term by term), then the mass step (finish).
 // src: component 0 of the other coset; (za, zb), (ya, yb), (xa, xb): its cells for h = +1 and
 // h = -1 per axis, with pitches sz (z) and sy (y); own: component 0 of the own cell.
 template <bool NC, typename C, typename CF, typename I>
 __device__ __forceinline__ void core_3d(const C* src, I sz, I sy, I za, I zb, I ya, I yb, I xa, I xb, I cs,
                                         const C* own, C (&r)[4], const CF& cf) {
-  C S0, S1, S2, S3;
-  {  // h_z = +1: plane za, components a, b, d
-    const C* pp = src + za * sz + ya * sy + xa;  // (h_x, h_y) = (+, +)
-    const C* pm = src + za * sz + yb * sy + xa;  // (+, -)
-    const C* mp = src + za * sz + ya * sy + xb;  // (-, +)
-    const C* mm = src + za * sz + yb * sy + xb;  // (-, -)
-    const C app = ldg<NC>(pp), bpp = ldg<NC>(pp + cs), dpp = ldg<NC>(pp + 3 * cs);
-    const C apm = ldg<NC>(pm), bpm = ldg<NC>(pm + cs), dpm = ldg<NC>(pm + 3 * cs);
-    const C amp = ldg<NC>(mp), bmp = ldg<NC>(mp + cs), dmp = ldg<NC>(mp + 3 * cs);
-    const C amm = ldg<NC>(mm), bmm = ldg<NC>(mm + cs), dmm = ldg<NC>(mm + 3 * cs);
-    S0 = cadd(rhob(cadd(cadd(app, bpp), csub(amm, bmm))), rho(cadd(cadd(apm, bpm), csub(amp, bmp))));
-    S2 = cadd(rhob(csub(dmm, dpp)), rho(csub(dmp, dpm)));
-    S3 = cadd(rhob(cadd(dpp, dmm)), rho(cadd(dpm, dmp)));
-  }
-  {  // h_z = -1: plane zb, components a, b, c
-    const C* pp = src + zb * sz + ya * sy + xa;
-    const C* pm = src + zb * sz + yb * sy + xa;
-    const C* mp = src + zb * sz + ya * sy + xb;
-    const C* mm = src + zb * sz + yb * sy + xb;
-    const C app = ldg<NC>(pp), bpp = ldg<NC>(pp + cs), cpp = ldg<NC>(pp + 2 * cs);
-    const C apm = ldg<NC>(pm), bpm = ldg<NC>(pm + cs), cpm = ldg<NC>(pm + 2 * cs);
-    const C amp = ldg<NC>(mp), bmp = ldg<NC>(mp + cs), cmp = ldg<NC>(mp + 2 * cs);
-    const C amm = ldg<NC>(mm), bmm = ldg<NC>(mm + cs), cmm = ldg<NC>(mm + 2 * cs);
-    S1 = cadd(rho(cadd(cadd(app, bpp), csub(bmm, amm))), rhob(cadd(cadd(apm, bpm), csub(bmp, amp))));
-    S2 = cadd(S2, cadd(rho(cadd(cpp, cmm)), rhob(cadd(cpm, cmp))));
-    S3 = cadd(S3, cadd(rho(csub(cmm, cpp)), rhob(csub(cmp, cpm))));
-  }
+  const C* app = src + za * sz + ya * sy + xa;  // plane of h_z = +1: (h_x, h_y) = (+, +)
+  const C* apm = src + za * sz + yb * sy + xa;  // (+, -)
+  const C* amp = src + za * sz + ya * sy + xb;  // (-, +)
+  const C* amm = src + za * sz + yb * sy + xb;  // (-, -)
+  const C* bpp = src + zb * sz + ya * sy + xa;  // plane of h_z = -1
+  const C* bpm = src + zb * sz + yb * sy + xa;
+  const C* bmp = src + zb * sz + ya * sy + xb;
+  const C* bmm = src + zb * sz + yb * sy + xb;
+  auto xsum = [&](const C* p) { return cadd(ldg<NC>(p), ldg<NC>(p + cs)); };
+  auto xdif = [&](const C* p) { return csub(ldg<NC>(p), ldg<NC>(p + cs)); };
+  const C S0 = rhob(addi(addi(xsum(app), xdif(amp)), subi(xsum(apm), xdif(amm))));
+  const C S1 = rho(subi(addi(xsum(bpp), xdif(bmp)), subi(xsum(bpm), xdif(bmm))));
+  auto v = [&](const C* c, const C* d) { return addi(ldg<NC>(c + 2 * cs), ldg<NC>(d + 3 * cs)); };
+  auto w = [&](const C* c, const C* d) { return subi(ldg<NC>(c + 2 * cs), ldg<NC>(d + 3 * cs)); };
+  const C G = rho(subi(v(bpp, app), w(bpm, apm)));
+  const C H = rhob(addi(v(bmp, amp), w(bmm, amm)));
   const C o0 = ldg<NC>(own), o1 = ldg<NC>(own + cs), o2 = ldg<NC>(own + 2 * cs), o3 = ldg<NC>(own + 3 * cs);
   r[0] = finish(cf, S0, o2);
   r[1] = finish(cf, S1, o3);
-  r[2] = finish(cf, S2, o0);
-  r[3] = finish(cf, S3, o1);
+  r[2] = finish(cf, cadd(H, G), o0);
+  r[3] = finish(cf, csub(H, G), o1);
 }
 
 template <typename R, bool NC = true, typename I = int64_t>
