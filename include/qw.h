@@ -64,9 +64,8 @@ typedef enum { QW_C64 = 0, QW_C128 = 1 } qw_dtype;
  * remaining step runs as TMA).  FUSED: any lattice and size, complex64; box
  * tiles of the field with a halo loaded into shared memory, `depth` steps per
  * launch (temporal fusion of depth 2..4, tile box and depth set by
- * qw_plan_set_fusion or the autotuner).  AUTO restores the default, the
- * fastest measured on GB300: FUSED for complex64 chains, else PLAIN;
- * qw_plan_autotune measures every variant (FUSED with
+ * qw_plan_set_fusion or the autotuner).  AUTO restores the default, PLAIN, the
+ * fastest measured on GB300; qw_plan_autotune measures every variant (FUSED with
  * several depths and boxes) and keeps the fastest. */
 typedef enum {
   QW_STENCIL_AUTO = 0,

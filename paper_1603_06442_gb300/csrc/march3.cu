@@ -29,8 +29,7 @@ qw_status launch_tile(const March3<typename CplxOf<R>::T>& p, int grid, typename
   constexpr int smem = march3_smem<R, KX, KY, NW>();
   const qw_status s = smem_attr(k, smem);
   if (s != QW_OK) return s;
-  k<<<grid, 32 * NW, smem, st>>>(p, cf);
-  QW_CHECK_LAUNCH("marching stencil launch");
+  QW_CHECK_CUDA(launch_overlapped(k, (unsigned)grid, 32 * NW, smem, st, p, cf));
   return QW_OK;
 }
 
@@ -67,7 +66,7 @@ double estimate3(const Geometry& g, const Tile3& s, int sms) {
   const int P = 2 * p.M;
   int iters = p.rounds * (P + 2 * s.t);
   if (p.rest) iters += (p.planes < P ? p.planes : P) + 2 * s.t;
-  return 4.0 + iters * s.us;  // us a launch: start and end, and the half-layers of the longest CTA
+  return 2.5 + iters * s.us;  // us a launch: start and end, and the half-layers of the longest CTA
 }
 
 }  // namespace

@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(32 * NW, CTAS)
         for (int q = 0; q < 4; ++q) L[t].own[y][k][q] = held<0>(C{0, 0});
       }
 
+  grid_wait();
   // the CTA's segments [ls, le) of a tile
   const int main_ctas = p.rest * p.per, b = blockIdx.x, tail = P - p.per * p.planes;
   int64_t pos = (int64_t)(b - main_ctas) * p.extra;  // in the remaining tiles' tails, one after another

@@ -1,5 +1,6 @@
 """The marching stencil kernels behind PLAIN (several steps per launch, the steps between held in
-registers) at the sizes where their tiles end: boxes around the tiles' widths, heights and chunks, and step counts that leave every remainder.
+registers) at the sizes where their windows and tiles end: chains around the lengths of a window,
+boxes around the tiles' widths, heights and chunks, and step counts that leave every remainder.
 
 They apply the per-site update in the same order, so complex64 fields equal FUSED's (box tiles in
 shared memory) bit for bit; complex128 has one per-site kernel, qw_step_static's.
@@ -30,7 +31,9 @@ def field(dim, N, dtype):
     return torch.randn(inputs.field_shape(dim, N), dtype=td, device="cuda", generator=g)
 
 
-SIZES = [(3, n) for n in (2, 4, 18, 20, 26, 40, 42, 56, 58, 64, 66, 96, 130, 250)]
+SIZES = [(1, n) for n in (2, 3, 31, 33, 63, 65, 127, 480, 481, 513, 1023, 20011)] + \
+        [(2, n) for n in (2, 3, 27, 28, 29, 56, 57, 61, 64, 65, 130, 301)] + \
+        [(3, n) for n in (2, 4, 18, 20, 26, 40, 42, 56, 58, 64, 66, 96, 130, 250)]
 
 
 @pytest.mark.parametrize("dim,N", SIZES)
@@ -46,7 +49,7 @@ def test_c64_equals_fused_bit_for_bit(qb, dim, N):
     plan.close()
 
 
-@pytest.mark.parametrize("dim,N", [(d, n) for d, n in SIZES if n < 250])
+@pytest.mark.parametrize("dim,N", [(d, n) for d, n in SIZES if n < 250 or d == 1])
 def test_c128_equals_the_per_site_kernel_bit_for_bit(qb, dim, N):
     plan = qb.Plan(dim, N, 0.27, "c128")
     for t in (1, 2, 5, 14, 67):
@@ -58,7 +61,7 @@ def test_c128_equals_the_per_site_kernel_bit_for_bit(qb, dim, N):
 
 
 @pytest.mark.parametrize("dtype", ["c64", "c128"])
-@pytest.mark.parametrize("dim,N", [(3, 44)])
+@pytest.mark.parametrize("dim,N", [(1, 97), (2, 31), (3, 44)])
 def test_marching_matches_the_oracle(qb, dtype, dim, N):
     m, t = 0.31, 23
     a = inputs.random_field(dim, N, seed=N)
