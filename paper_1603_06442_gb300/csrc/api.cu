@@ -150,7 +150,7 @@ bool make_geometry(int dim, int64_t N, Geometry* g) {
 
 static int default_stencil(const qw_plan_s* p) {
   // the marching kernels behind PLAIN are the fastest measured on every lattice, size and type
-  // (march1.cu, march3.cu); qw_plan_autotune re-measures on the device
+  // (march1.cu, march2.cu, march3.cu); qw_plan_autotune re-measures on the device
   (void)p;
   return QW_STENCIL_PLAIN;
 }
@@ -339,21 +339,23 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     QW_CHECK_CUDA(cudaMemsetAsync(p->scratch, kPoisonByte, (size_t)p->g.elems * p->elem_bytes, s));
   void* cur = psi;
   void* nxt = p->scratch;
-  int64_t march[5] = {0, 0, 0, 0, 0};  // PLAIN on BCC boxes: launches of 1..4 steps left
-  const bool marching = variant == QW_STENCIL_PLAIN && p->g.dim == 3;
-  if (marching) march3_schedule(p->g, p->dtype, nsteps, p->sms, march);
+  int64_t march[5] = {0, 0, 0, 0, 0};  // PLAIN on the square lattice and BCC boxes: launches of 1..4 steps left
+  const bool marching = variant == QW_STENCIL_PLAIN && march_supported(p->g, p->dtype);
+  if (marching) march_schedule(p->g, p->dtype, nsteps, p->sms, march);
   March1 chain{0, 0};  // PLAIN on the chain: launches left
   if (variant == QW_STENCIL_PLAIN && p->g.dim == 1) chain = march1_schedule(p->g.nx, p->dtype, nsteps, p->sms);
+  int last = 0;  // steps of the launch before: the same kernel again may start while it drains
   for (int64_t i = 0; i < nsteps;) {
     int done = 1;
     if (marching) {
       done = march[4] ? 4 : march[3] ? 3 : march[2] ? 2 : 1;
       --march[done];
-      st = launch_march3(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, s);
+      st = p->g.dim == 2 ? launch_march2(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, done == last, s)
+                         : launch_march3(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, done == last, s);
     } else if (chain.launches > 0) {
       done = (int)((nsteps - i + chain.launches - 1) / chain.launches);
       --chain.launches;
-      st = launch_march1(p->g.nx, p->dtype, chain.K, done, p->n, p->mass, cur, nxt, p->sms, s);
+      st = launch_march1(p->g.nx, p->dtype, chain.K, done, p->n, p->mass, cur, nxt, p->sms, last > 0, s);
     } else if (variant == QW_STENCIL_TMA2 && nsteps - i >= 2) {
       st = launch_step_tma2(p->g, p->n, p->mass, cur, nxt, p->tma2_items, p->tma2_nitems, p->dev_flags,
                             p->dev_flags + 1, s);
@@ -372,6 +374,7 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     cur = nxt;
     nxt = t;
     i += done;
+    last = done;
   }
   if (cur != psi)
     QW_CHECK_CUDA(cudaMemcpyAsync(psi, cur, (size_t)p->g.elems * p->elem_bytes, cudaMemcpyDeviceToDevice, s));

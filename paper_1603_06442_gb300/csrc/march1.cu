@@ -111,14 +111,13 @@ template <typename R> double cost1(int64_t N, int K, int steps, int sms) {
 
 template <typename R, int K>
 qw_status launch1(const void* in, void* out, int64_t N, int steps, typename CoefOf<R>::T cf, int sms,
-                  cudaStream_t st) {
+                  bool overlap, cudaStream_t st) {
   using C = typename CplxOf<R>::T;
   const int64_t windows = (N + 32 * K - 2 * steps - 1) / (32 * K - 2 * steps);
   // few windows: a warp per CTA, so that they spread over the SMs
   const int warps = windows < (int64_t)kWarps1 * sms ? 1 : kWarps1;
-  QW_CHECK_CUDA(launch_overlapped(march1d_kernel<R, K>, (unsigned)((windows + warps - 1) / warps), 32 * warps, 0, st,
-                                  static_cast<const C*>(in), static_cast<C*>(out), N, steps, windows, cf));
-  return QW_OK;
+  return launch_overlapped(march1d_kernel<R, K>, (unsigned)((windows + warps - 1) / warps), 32 * warps, 0, overlap,
+                           st, static_cast<const C*>(in), static_cast<C*>(out), N, steps, windows, cf);
 }
 
 }  // namespace
@@ -152,23 +151,23 @@ March1 march1_schedule(int64_t N, qw_dtype dt, int64_t nsteps, int sms) {
 }
 
 qw_status launch_march1(int64_t N, qw_dtype dt, int K, int steps, double n, double m, const void* in, void* out,
-                        int sms, cudaStream_t st) {
+                        int sms, bool overlap, cudaStream_t st) {
   if (dt == QW_C64) {
     const Coef32 cf = make_coef32(1, n, m);
     switch (K) {
-      case 1: return launch1<float, 1>(in, out, N, steps, cf, sms, st);
-      case 2: return launch1<float, 2>(in, out, N, steps, cf, sms, st);
-      case 4: return launch1<float, 4>(in, out, N, steps, cf, sms, st);
-      case 8: return launch1<float, 8>(in, out, N, steps, cf, sms, st);
-      default: return launch1<float, 16>(in, out, N, steps, cf, sms, st);
+      case 1: return launch1<float, 1>(in, out, N, steps, cf, sms, overlap, st);
+      case 2: return launch1<float, 2>(in, out, N, steps, cf, sms, overlap, st);
+      case 4: return launch1<float, 4>(in, out, N, steps, cf, sms, overlap, st);
+      case 8: return launch1<float, 8>(in, out, N, steps, cf, sms, overlap, st);
+      default: return launch1<float, 16>(in, out, N, steps, cf, sms, overlap, st);
     }
   }
   const Coef64 cf = make_coef64(1, n, m);
   switch (K) {
-    case 1: return launch1<double, 1>(in, out, N, steps, cf, sms, st);
-    case 2: return launch1<double, 2>(in, out, N, steps, cf, sms, st);
-    case 4: return launch1<double, 4>(in, out, N, steps, cf, sms, st);
-    default: return launch1<double, 8>(in, out, N, steps, cf, sms, st);
+    case 1: return launch1<double, 1>(in, out, N, steps, cf, sms, overlap, st);
+    case 2: return launch1<double, 2>(in, out, N, steps, cf, sms, overlap, st);
+    case 4: return launch1<double, 4>(in, out, N, steps, cf, sms, overlap, st);
+    default: return launch1<double, 8>(in, out, N, steps, cf, sms, overlap, st);
   }
 }
 

@@ -1,0 +1,148 @@
+// The square lattice: several steps of the update rule per pass over HBM with the marching kernel of
+// qw_march2.cuh, the split of a field over its warps, and (for the BCC boxes too) the mix of launches
+// that makes a number of steps.
+//
+// complex64, one GB300: N = 2998, 150 steps: 7.03 ms against 15.3 ms of one thread per site and one
+// pass per step; G site-steps/s of the kernel: N = 8192: 263 (four steps a pass) against 94.  It is bound by the FP32 pipe
+// and issue (IPC 0.64; 41 additions, 16 packed mass operations and 4 shuffles a site-step), then by
+// the halo of 8 in 64 columns; HBM is at 40%.  Measured slower: rows handed from level to level one
+// row late, so that the levels are independent (253 at N = 8192), and the sums in packed additions
+// (244: fewer instructions, the same pipe).
+// One step, and complex128 (64 FP64 instructions a site-step on the FP64 pipe, where a recomputed
+// halo costs as much as shared sums save: 523 against 539 us at N = 2048), stay with one thread per
+// site (stencil.cu).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+
+#include "qw_march2.cuh"
+
+namespace qw {
+namespace {
+
+// Instantiated kernels: KX columns per lane, T steps, warps per CTA, CTAs per SM; us of one row with
+// the SM full, and of one row of a warp on its own (measured).
+struct Strip2 {
+  int kx, t, nw, ctas;
+  double full, own;
+};
+#define QW_STRIPS2(X) X(2, 4, 4, 2, 1.00, 0.45) X(2, 3, 4, 3, 1.25, 0.36) X(2, 2, 4, 4, 1.55, 0.27)
+#define X(kx, t, nw, ctas, full, own) {kx, t, nw, ctas, full, own},
+const Strip2 kStrips[] = {QW_STRIPS2(X)};
+#undef X
+
+// The chunks of rows per strip: enough warps for every SM, but no more rows recomputed at the chunks'
+// ends (2 T each) than the waves saved; *us receives the estimate of the launch.
+March2 geometry2(int64_t N, const Strip2& s, int sms, double* us) {
+  March2 p{};
+  p.N = (int)N;
+  p.tx = 32 * s.kx - 2 * s.t;
+  p.ntx = (p.N + p.tx - 1) / p.tx;
+  const int full = sms * s.ctas * s.nw;  // resident warps
+  const int base = std::max(1, full / p.ntx);
+  double best = -1.0;
+  for (int c : {1, base / 8, base / 4, base / 2, base, 2 * base, 3 * base, 4 * base, p.N}) {
+    if (c < 1 || c > p.N) continue;
+    const int rows = (p.N + c - 1) / c, chunks = (p.N + rows - 1) / rows;
+    const int64_t items = (int64_t)p.ntx * chunks;
+    const int64_t waves = (items + full - 1) / full;
+    // rows of the SM with most warps: full waves, or a part of one between the two measured ends
+    const double share = waves > 1 ? 1.0 : (double)((items + sms - 1) / sms) / (s.ctas * s.nw);
+    const double t = waves * (rows + 2 * s.t) * std::max(s.own, s.full * share);
+    if (best < 0 || t < best) {
+      best = t;
+      p.rows = rows;
+      p.chunks = chunks;
+    }
+  }
+  *us = 2.5 + best;
+  return p;
+}
+
+template <int KX, int T, int NW, int CTAS>
+qw_status launch_strips(const March2& p, const Coef32& cf, bool overlap, cudaStream_t st) {
+  auto* k = march2d_kernel<KX, T, NW, CTAS>;
+  constexpr int smem = march2_smem<KX, NW>();
+  const qw_status s = smem_attr(k, smem);
+  if (s != QW_OK) return s;
+  const int64_t items = (int64_t)p.ntx * p.chunks;
+  return launch_overlapped(k, (unsigned)((items + NW - 1) / NW), 32 * NW, smem, overlap, st, p, cf);
+}
+
+const Strip2* strip2(int steps) {
+  for (const Strip2& s : kStrips)
+    if (s.t == steps) return &s;
+  return nullptr;
+}
+
+}  // namespace
+
+double march2_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
+  // one thread per site: launches and HBM at 90 G site-steps/s (complex64), or the FP64 pipe
+  if (steps == 1) return 4.0 + (double)g.sites / (dt == QW_C64 ? 90.0e3 : 7.8e3);
+  const Strip2* s = dt == QW_C64 ? strip2(steps) : nullptr;
+  if (!s) return -1.0;
+  double us;
+  geometry2(g.nx, *s, sms, &us);
+  return us;
+}
+
+qw_status launch_march2(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
+                        int sms, bool overlap, cudaStream_t st) {
+  if (steps == 1) return launch_step(g, dt, QW_STENCIL_PLAIN, n, m, in, out, st);
+  const Strip2* s = dt == QW_C64 ? strip2(steps) : nullptr;
+  if (!s) {
+    set_error("marching stencil: no kernel for %d steps", steps);
+    return QW_EINVAL;
+  }
+  double us;
+  March2 p = geometry2(g.nx, *s, sms, &us);
+  for (int q = 0; q < 4; ++q) {
+    p.in[q] = static_cast<const float2*>(in) + q * g.vol;
+    p.out[q] = static_cast<float2*>(out) + q * g.vol;
+  }
+  const Coef32 cf = make_coef32(2, n, m);
+#define X(kx, T, nw, ctas, full, own) \
+  if (s->t == T) return launch_strips<kx, T, nw, ctas>(p, cf, overlap, st);
+  QW_STRIPS2(X)
+#undef X
+  return QW_EINVAL;
+}
+
+// The kernels index a component plane (of a coset) in 32 bits.
+bool march_supported(const Geometry& g, qw_dtype) { return g.dim >= 2 && g.vol < (int64_t)1 << 32; }
+
+// The cheapest mix by the estimates; an odd number of launches ends in the scratch field and costs a
+// copy of the field.
+void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]) {
+  double cost[5];
+  for (int t = 1; t <= 4; ++t) cost[t] = g.dim == 2 ? march2_cost(g, dt, t, sms) : march3_cost(g, dt, t, sms);
+  const double copy = 3.0 + 2.0 * (double)g.elems * (dt == QW_C64 ? 8 : 16) / 6.0e6;
+  double best = -1.0;
+  for (int64_t& c : count) c = 0;
+  // small counts of three of the sizes, the rest in launches of the fourth
+  for (int main = 1; main <= 4; ++main) {
+    if (cost[main] < 0) continue;
+    int64_t k[5] = {0, 0, 0, 0, 0};
+    const int a = main == 1 ? 2 : 1, b = main <= 2 ? 3 : 2, c = main <= 3 ? 4 : 3;
+    const int most[5] = {0, cost[1] < 0 ? 0 : 4, cost[2] < 0 ? 0 : 4, cost[3] < 0 ? 0 : 4, cost[4] < 0 ? 0 : 4};
+    for (k[a] = 0; k[a] <= most[a]; ++k[a])
+      for (k[b] = 0; k[b] <= most[b]; ++k[b])
+        for (k[c] = 0; k[c] <= most[c]; ++k[c]) {
+          const int64_t left = nsteps - a * k[a] - b * k[b] - c * k[c];
+          if (left < 0 || left % main) continue;
+          k[main] = left / main;
+          const int64_t launches = k[1] + k[2] + k[3] + k[4];
+          double total = launches % 2 ? copy : 0.0;
+          for (int t = 1; t <= 4; ++t)
+            if (k[t]) total += (double)k[t] * cost[t];
+          if (best < 0 || total < best) {
+            best = total;
+            for (int t = 1; t <= 4; ++t) count[t] = k[t];
+          }
+        }
+    k[main] = 0;
+  }
+}
+
+}  // namespace qw

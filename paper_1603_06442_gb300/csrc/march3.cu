@@ -24,13 +24,13 @@ struct Tile3 {
   double us;
 };
 template <typename R, int KX, int KY, int T, int NW, int CTAS>
-qw_status launch_tile(const March3<typename CplxOf<R>::T>& p, int grid, typename CoefOf<R>::T cf, cudaStream_t st) {
+qw_status launch_tile(const March3<typename CplxOf<R>::T>& p, int grid, typename CoefOf<R>::T cf, bool overlap,
+                      cudaStream_t st) {
   auto* k = march3d_kernel<R, KX, KY, T, NW, CTAS>;
   constexpr int smem = march3_smem<R, KX, KY, NW>();
   const qw_status s = smem_attr(k, smem);
   if (s != QW_OK) return s;
-  QW_CHECK_CUDA(launch_overlapped(k, (unsigned)grid, 32 * NW, smem, st, p, cf));
-  return QW_OK;
+  return launch_overlapped(k, (unsigned)grid, 32 * NW, smem, overlap, st, p, cf);
 }
 
 #define QW_TILES3_C64(X)                                                                            \
@@ -71,7 +71,6 @@ double estimate3(const Geometry& g, const Tile3& s, int sms) {
 
 }  // namespace
 
-// us of a launch of `steps` steps (the best tile for it), or < 0 where no tile takes that many.
 double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
   double best = -1.0;
   const Tile3* t = dt == QW_C64 ? kTiles64 : kTiles128;
@@ -84,40 +83,8 @@ double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
   return best;
 }
 
-// Launches of 4, 3, 2 and 1 steps that make nsteps: the cheapest mix by the estimates above; an odd
-// number of launches ends in the scratch field and costs a copy of the field.
-void march3_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]) {
-  double cost[5];
-  for (int t = 1; t <= 4; ++t) cost[t] = march3_cost(g, dt, t, sms);
-  const double copy = 3.0 + 2.0 * (double)g.elems * (dt == QW_C64 ? 8 : 16) / 6.0e6;
-  double best = -1.0;
-  for (int64_t& c : count) c = 0;
-  // small counts of three of the sizes, the rest in launches of the fourth
-  for (int main = 1; main <= 4; ++main) {
-    if (cost[main] < 0) continue;
-    int64_t k[5] = {0, 0, 0, 0, 0};
-    const int a = main == 1 ? 2 : 1, b = main <= 2 ? 3 : 2, c = main <= 3 ? 4 : 3;
-    for (k[a] = 0; k[a] <= 4; ++k[a])
-      for (k[b] = 0; k[b] <= 4; ++k[b])
-        for (k[c] = 0; k[c] <= 4; ++k[c]) {
-          if ((k[a] && cost[a] < 0) || (k[b] && cost[b] < 0) || (k[c] && cost[c] < 0)) continue;
-          const int64_t left = nsteps - a * k[a] - b * k[b] - c * k[c];
-          if (left < 0 || left % main) continue;
-          k[main] = left / main;
-          const int64_t launches = k[1] + k[2] + k[3] + k[4];
-          double total = launches % 2 ? copy : 0.0;
-          for (int t = 1; t <= 4; ++t)
-            if (k[t]) total += (double)k[t] * cost[t];
-          if (best < 0 || total < best) {
-            best = total;
-            for (int t = 1; t <= 4; ++t) count[t] = k[t];
-          }
-        }
-  }
-}
-
 qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
-                        int sms, cudaStream_t st) {
+                        int sms, bool overlap, cudaStream_t st) {
   const Tile3* t = dt == QW_C64 ? kTiles64 : kTiles128;
   const int cnt = dt == QW_C64 ? (int)(sizeof(kTiles64) / sizeof(Tile3)) : (int)(sizeof(kTiles128) / sizeof(Tile3));
   int best = -1;
@@ -148,7 +115,7 @@ qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, dou
     planes(p);
     const Coef32 cf = make_coef32(3, n, m);
 #define X(kx, ky, T, nw, ctas, us) \
-  if (i++ == best) return launch_tile<float, kx, ky, T, nw, ctas>(p, grid, cf, st);
+  if (i++ == best) return launch_tile<float, kx, ky, T, nw, ctas>(p, grid, cf, overlap, st);
     QW_TILES3_C64(X)
   } else {
     March3<double2> p = geometry3<double2>(g, t[best], sms, &grid);
@@ -156,7 +123,7 @@ qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, dou
     const Coef64 cf = make_coef64(3, n, m);
 #undef X
 #define X(kx, ky, T, nw, ctas, us) \
-  if (i++ == best) return launch_tile<double, kx, ky, T, nw, ctas>(p, grid, cf, st);
+  if (i++ == best) return launch_tile<double, kx, ky, T, nw, ctas>(p, grid, cf, overlap, st);
     QW_TILES3_C128(X)
 #undef X
   }

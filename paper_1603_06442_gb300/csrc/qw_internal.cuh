@@ -53,18 +53,17 @@ inline int resident_blocks(K* kernel, int threads, int smem = 0) {
     if (qw_e_ != cudaSuccess) return ::qw::cuda_fail(qw_e_, what);  \
   } while (0)
 
-template <typename T> struct CplxOf2;
-template <> struct CplxOf2<float> { using t = float2; };
-template <> struct CplxOf2<double> { using t = double2; };
-
 // Launch that may start while the stream's previous kernel drains (programmatic stream
 // serialisation): the kernel calls grid_wait() before its first access to global memory, which
 // returns when every earlier kernel of the stream has completed and its writes are visible.  A
 // dependent launch then costs 1.4 us instead of 2.1 to 4.1 on GB300 (a kernel's end is otherwise
-// noticed at intervals of about 2 us).  Needs no more of the previous kernel than its launch.
+// noticed at intervals of about 2 us).  overlap = false is a plain launch: for a kernel other than
+// the previous one.  An SM changes its split of L1 and shared memory only when it is empty, and a
+// kernel that overlaps another one's end keeps that one's split, also for the launches after it:
+// a third slower where it leaves less L1 for the loads in flight (square lattice, N = 2998).
 template <typename... P, typename... A>
-inline cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, int smem, cudaStream_t st,
-                                     A... args) {
+inline qw_status launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, int smem, bool overlap,
+                                   cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(grid);
   cfg.blockDim = dim3(block);
@@ -74,8 +73,9 @@ inline cudaError_t launch_overlapped(void (*kernel)(P...), unsigned grid, unsign
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+  cfg.numAttrs = overlap ? 1 : 0;
+  QW_CHECK_CUDA(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
+  return QW_OK;
 }
 #ifdef __CUDACC__
 __device__ __forceinline__ void grid_wait() {
@@ -84,6 +84,10 @@ __device__ __forceinline__ void grid_wait() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 #endif
+
+template <typename T> struct CplxOf2;
+template <> struct CplxOf2<float> { using t = float2; };
+template <> struct CplxOf2<double> { using t = double2; };
 
 // ---- debug poison (api.cu): while on, scratch and partner buffers are filled with NaN
 // (all bytes 0xFF) before each call that must write them before reading them
@@ -147,11 +151,18 @@ qw_status launch_step_tma2(const Geometry& g, double n, double m, const void* in
                            int nitems, int* err, int* next_item, cudaStream_t st);
 qw_status launch_step_tma(const Geometry& g, double n, double m, const void* in, void* out, const int4* items,
                           int nitems, int* err, int* next_item, cudaStream_t st);
-// Marching kernels, BCC (march3.cu): `steps` updates out = U^steps in per launch, the steps between held
-// in registers.  march3_schedule: how many launches of 1..4 steps make nsteps.
-void march3_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]);
+// Marching kernels (march2.cu: square lattice, march3.cu: BCC): `steps` (1..4) updates
+// out = U^steps in per launch, the steps between held in registers.  The costs are estimates in us
+// of one launch, < 0 where no kernel takes that many steps; march_schedule: how many launches of
+// 1..4 steps make nsteps.
+bool march_supported(const Geometry& g, qw_dtype dt);
+double march2_cost(const Geometry& g, qw_dtype dt, int steps, int sms);
+double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms);
+void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]);
+qw_status launch_march2(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
+                        int sms, bool overlap, cudaStream_t st);
 qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
-                        int sms, cudaStream_t st);
+                        int sms, bool overlap, cudaStream_t st);
 // The chain (march1.cu): `launches` launches with K sites per lane make nsteps steps.
 struct March1 {
   int K;
@@ -159,7 +170,7 @@ struct March1 {
 };
 March1 march1_schedule(int64_t N, qw_dtype dt, int64_t nsteps, int sms);
 qw_status launch_march1(int64_t N, qw_dtype dt, int K, int steps, double n, double m, const void* in, void* out,
-                        int sms, cudaStream_t st);
+                        int sms, bool overlap, cudaStream_t st);
 // FUSED: `steps` <= depth updates in one launch, box tiles of the field and a halo in shared
 // memory (complex64, any geometry whose tile fits shared memory; batch.cu).
 bool fused_step_supported(const Geometry& g, qw_dtype dt, int depth, const int* box);
