@@ -8,7 +8,11 @@
 // (r + 1) % 2; when the number of stepping rounds is odd a last round copies
 // the result back into the caller's field.  The fusion depth T_w is set per
 // lattice dimension:
-//   * T = 1: each cell is updated from global memory (the plain per-site update);
+//   * T = 1, when no walk of the batch is fused: marching rounds of the square lattice (four
+//     steps) and BCC boxes (three) with the steps between held in registers (qw_march.cuh,
+//     qw_march2.cuh), the steps left over one per round.  The 256-walk mix on one GB300: 132 ms
+//     against 307 ms of per-site rounds (161 against 69 G site-steps/s);
+//   * T = 1 else, and on the chain: each cell is updated from global memory (the per-site update);
 //   * T >= 2 (temporal fusion): the tile and a halo of H cells per side (H = T on
 //     the chain and the square lattice, ceil(T/2) on the BCC lattice, where one
 //     step reaches one cell of the other coset) are copied into shared memory by
@@ -40,13 +44,16 @@
 #include <vector>
 
 #include "qw_internal.cuh"
+#include "qw_march2.cuh"
 #include "qw_stencil_dev.cuh"
 
 namespace qw {
 
 struct BatchWalk {
   int dim;
-  int depth;          // steps per round: 1 = per-site update from global memory, >= 2 = fused
+  int depth;          // steps per stepping round
+  int march;          // rounds run in the marching kernels' registers (square lattice, BCC)
+  int64_t nfull;      // marching rounds (depth steps each); the steps left follow one per round
   int halo;           // H: cells per side beyond the tile that one round depends on
   int ncos, ncomp;    // cosets (2 on the BCC lattice) and spinor components
   int n[3];           // cells per axis (nx, ny, nz)
@@ -56,7 +63,7 @@ struct BatchWalk {
   int vol;            // cells of one coset-component plane (walks hold < 2^31 values)
   int64_t tile_base;  // first entry of this walk in the per-tile round counters
   int64_t t;          // steps per run
-  int64_t nstep;      // stepping rounds: ceil(t / depth)
+  int64_t nstep;      // stepping rounds
   int64_t rounds;     // nstep, plus one copy round when nstep is odd
   float2* buf[2];     // buf[0] = caller's field, buf[1] = partner
   Coef32 cf;
@@ -86,10 +93,12 @@ struct BatchDebug {
 };
 
 constexpr long long kBatchSpin = 1ll << 24;
-constexpr int kBatchThreads = 256;   // plain (depth-1) launches
-// plain launches: CTAs per SM the register budget is cut for (64 registers, no spills; 6 and 3
-// CTAs, and cells taken two at a time, measured 2-15% slower on the uneven 256-walk mix)
-constexpr int kBatchMinBlocks = 4;
+// Marching launches (no walk fused in shared memory): four warps, two CTAs per SM.  A square-lattice
+// item is a strip of kCols columns and four warps' rows, kT2 steps; a BCC item a tile of
+// tile3_geo(M, 1, kRows3, kT3, 4) and a chunk of layers, kT3 steps.
+constexpr int kMarchThreads = 128, kT2 = 4, kCols = 64 - 2 * kT2, kT3 = 3, kRows3 = 3;
+constexpr int kMarchSmem = march2_smem<2, 4>() > march3_smem<float, 1, kRows3, 4>() ? march2_smem<2, 4>()
+                                                                                   : march3_smem<float, 1, kRows3, 4>();
 constexpr int kFusedThreads = 256;   // launches with fused rounds (512 measured slower: 172 vs 232 G on the chain)
 
 // Largest i in [0, n) with a[i] <= v (a ascending, a[0] <= v), searched by the 32 lanes
@@ -324,15 +333,36 @@ __device__ __forceinline__ void plain_round(const BatchWalk& W, const int (&t3)[
   }
 }
 
-// FUSED = false: every walk has depth 1 (no shared memory, high occupancy);
-// FUSED = true: walks of depth >= 2 run fused rounds in dynamic shared memory.
+// A marching round of tile (t0, t1, t2): depth steps of the tile, from in to out.
+__device__ __forceinline__ void march_round(const BatchWalk& W, const int (&t3)[3], const float2* in, float2* out,
+                                            unsigned char* smem) {
+  const CoefF2 cf = spread(W.cf);
+  if (W.dim == 2) {
+    const int rows = W.ext[1] / 4, N = W.n[0];
+    const int ys = t3[1] * W.ext[1] + (int)(threadIdx.x >> 5) * rows;
+    if (ys < N)
+      march2_rows<2, kT2, 4, true>(
+          N, t3[0], ys, min(ys + rows, N), smem, [&](int q) { return in + q * W.vol; },
+          [&](int q) { return out + q * W.vol; }, cf);
+  } else {
+    const int ls = 2 * t3[2] * W.ext[2], le = min(ls + 2 * W.ext[2], 2 * W.n[2]);
+    march3_segment<float, 1, kRows3, kT3, 4, true>(
+        tile3_geo(W.n[0], 1, kRows3, kT3, 4), t3[0], t3[1], ls, le, smem,
+        [&](int c, int q) { return in + (c * 4 + q) * W.vol; }, [&](int c, int q) { return out + (c * 4 + q) * W.vol; },
+        cf);
+  }
+}
+
+// FUSED = false: walks of the square lattice and BCC boxes run marching rounds, chains per-site
+// rounds; FUSED = true: walks of depth >= 2 run fused rounds in dynamic shared memory, the others
+// per-site rounds.
 template <bool FUSED>
-__global__ void __launch_bounds__(FUSED ? kFusedThreads : kBatchThreads, FUSED ? 3 : kBatchMinBlocks)
+__global__ void __launch_bounds__(FUSED ? kFusedThreads : kMarchThreads, FUSED ? 3 : 2)
     batch_kernel(const BatchWalk* __restrict__ walks, const BatchGroup* __restrict__ groups,
                  const int64_t* __restrict__ group_item0, int ngroups, const int64_t* __restrict__ tile_prefix,
                  const int64_t* __restrict__ round_prefix, int64_t total_items, unsigned int* __restrict__ done,
                  BatchCtl* __restrict__ ctl, BatchDebug dbg) {
-  extern __shared__ float2 smem_dyn[];
+  extern __shared__ __align__(16) float2 smem_dyn[];
   __shared__ int64_t s_next, s_round;
   __shared__ int s_abort, s_walk, s_tile;
   const int tid = threadIdx.x;
@@ -428,16 +458,23 @@ __global__ void __launch_bounds__(FUSED ? kFusedThreads : kBatchThreads, FUSED ?
     if (s < W.nstep) {
       const float2* in = (s & 1) ? b1 : b0;
       float2* out = (s & 1) ? b0 : b1;
-      const int steps = (int)min((int64_t)W.depth, W.t - s * W.depth);
-      if (FUSED && W.depth > 1) {
-        const int P = (W.ncos * W.ncomp) * (W.ext[0] + 2 * W.halo) * (W.dim >= 2 ? W.ext[1] + 2 * W.halo : 1) *
-                      (W.dim >= 3 ? W.ext[2] + 2 * W.halo : 1);
-        fused_round<FUSED ? kFusedThreads : kBatchThreads>(W, t3, steps, in, out, smem_dyn, smem_dyn + P);
-      } else {
-        plain_round<FUSED ? kFusedThreads : kBatchThreads>(W, t3, false, in, out);
+      constexpr int NT = FUSED ? kFusedThreads : kMarchThreads;
+      bool done_round = false;
+      if constexpr (FUSED) {
+        if (W.depth > 1) {
+          const int steps = (int)min((int64_t)W.depth, W.t - s * W.depth);
+          const int P = (W.ncos * W.ncomp) * (W.ext[0] + 2 * W.halo) * (W.dim >= 2 ? W.ext[1] + 2 * W.halo : 1) *
+                        (W.dim >= 3 ? W.ext[2] + 2 * W.halo : 1);
+          fused_round<NT>(W, t3, steps, in, out, smem_dyn, smem_dyn + P);
+          done_round = true;
+        }
+      } else if (s < W.nfull) {
+        march_round(W, t3, in, out, reinterpret_cast<unsigned char*>(smem_dyn));
+        done_round = true;
       }
+      if (!done_round) plain_round<NT>(W, t3, false, in, out);
     } else {
-      plain_round<FUSED ? kFusedThreads : kBatchThreads>(W, t3, true, b1, b0);  // copy round: the result sits in buf[1]
+      plain_round<FUSED ? kFusedThreads : kMarchThreads>(W, t3, true, b1, b0);  // copy round: the result sits in buf[1]
     }
     __syncthreads();
     if (tid == 0 && W.tile_base + tile != dbg.stall_tile) {
@@ -500,8 +537,8 @@ struct qw_batch_s {
 
 namespace qw {
 
-// Defaults: what the autotuner picks for the 256-walk mix on GB300 (depth 1 on every lattice,
-// 2048-site rows, one group); the boxes are those of fused rounds when a depth is raised.
+// Defaults: the fastest measured for the 256-walk mix on GB300 (depth 1 on every lattice: marching
+// rounds; 2048-site tiles on the chain, one group); the boxes are those of fused rounds when a depth is raised.
 static qw_batch_tiling default_tiling() {
   qw_batch_tiling t;
   t.tile_sites = 2048;
@@ -573,8 +610,9 @@ static int64_t field_bytes(const qw_walk& w) {
   return g.elems * 8;
 }
 
-// The walk's entry of the schedule under tiling t (tiles, depth, rounds).
-static BatchWalk make_walk(const qw_walk& d, void* partner, const qw_batch_tiling& t) {
+// The walk's entry of the schedule under tiling t (tiles, depth, rounds); march: a depth of 1 on the
+// square lattice and BCC boxes means marching rounds (no walk of the launch is fused).
+static BatchWalk make_walk(const qw_walk& d, void* partner, const qw_batch_tiling& t, bool march) {
   Geometry g;
   make_geometry(d.dim, d.N, &g);
   BatchWalk W;
@@ -585,7 +623,22 @@ static BatchWalk make_walk(const qw_walk& d, void* partner, const qw_batch_tilin
   W.n[0] = (int)g.nx;
   W.n[1] = (int)g.ny;
   W.n[2] = (int)g.nz;
-  if (W.depth == 1) {
+  W.march = march && d.dim >= 2;
+  if (W.march && d.dim == 2) {
+    // 64 rows a warp (an eighth more is recomputed at their ends), fewer where the walk has fewer
+    const int rows = std::min(64, std::max(8, (W.n[1] + 3) / 4));
+    W.depth = W.halo = kT2;
+    W.ext[0] = kCols;
+    W.ext[1] = 4 * rows;
+    W.ext[2] = 1;
+  } else if (W.march) {
+    const Tile3Geo tile = tile3_geo(W.n[0], 1, kRows3, kT3, 4);
+    W.depth = kT3;
+    W.halo = (kT3 + 1) / 2;
+    W.ext[0] = tile.tx;
+    W.ext[1] = tile.ty;
+    W.ext[2] = std::min(32, W.n[2]);  // 2 kT3 of 64 half-layers are recomputed
+  } else if (W.depth == 1) {
     // whole x rows (x segments on the chain), about tile_sites sites per tile
     W.halo = 1;
     if (d.dim == 1) {
@@ -608,7 +661,8 @@ static BatchWalk make_walk(const qw_walk& d, void* partner, const qw_batch_tilin
   }
   W.vol = (int)g.vol;
   W.t = d.t;
-  W.nstep = (d.t + W.depth - 1) / W.depth;
+  W.nfull = W.march ? d.t / W.depth : 0;
+  W.nstep = W.march ? W.nfull + d.t % W.depth : (d.t + W.depth - 1) / W.depth;
   W.rounds = W.nstep + (W.nstep & 1);
   W.buf[0] = static_cast<float2*>(d.psi_dev);
   W.buf[1] = static_cast<float2*>(partner);
@@ -642,7 +696,7 @@ qw_status launch_step_fused(const Geometry& g, int depth, const int* box, int st
   qw_batch_tiling t = default_tiling();
   t.depth[g.dim - 1] = depth;
   for (int a = 0; a < 3; ++a) t.box[g.dim - 1][a] = box[a];
-  BatchWalk W = make_walk(d, out, t);
+  BatchWalk W = make_walk(d, out, t, false);
   W.cf = make_coef32(g.dim, n, m);
   const size_t smem = fused_smem(W.dim, W.depth, W.ext);
   qw_status sa = smem_attr(fused_step_kernel, (int)smem);
@@ -683,13 +737,15 @@ static qw_status build_schedule(qw_batch_s* b) {
   std::vector<int64_t> tiles, rounds;
   b->order.clear();
   b->first_tile.assign(n, 0);
-  b->fused = false;
-  b->smem = 0;
+  bool fused = false;
+  for (const qw_walk& d : b->desc) fused = fused || b->tiling.depth[d.dim - 1] > 1;
+  b->fused = fused;
+  b->smem = fused ? 0 : kMarchSmem;
   int64_t item0 = 0;
   int64_t ndone_acc = 0;
   for (auto& gw : grp) {
     std::vector<BatchWalk> gwalks;
-    for (int i : gw) gwalks.push_back(make_walk(b->desc[i], b->partners[i], b->tiling));
+    for (int i : gw) gwalks.push_back(make_walk(b->desc[i], b->partners[i], b->tiling, !fused));
     // inside a group: most rounds first, so the walks alive at round s are a prefix
     std::vector<int> ord(gw.size());
     for (size_t k = 0; k < gw.size(); ++k) ord[k] = (int)k;
@@ -707,7 +763,7 @@ static qw_status build_schedule(qw_batch_s* b) {
       W.tile_base = ndone_acc;
       b->first_tile[gw[k]] = ndone_acc;
       ndone_acc += W.ntiles;
-      if (W.depth > 1) {
+      if (fused && W.depth > 1) {
         // the box clipped to the walk: a box larger than a small walk costs nothing extra
         const size_t need = fused_smem(W.dim, W.depth, W.ext);
         if (need > kMaxBatchSmem) {
@@ -715,7 +771,6 @@ static qw_status build_schedule(qw_batch_s* b) {
                     W.dim, W.depth, need, kMaxBatchSmem);
           return QW_EINVAL;
         }
-        b->fused = true;
         b->smem = std::max(b->smem, need);
       }
       walks.push_back(W);
@@ -769,7 +824,10 @@ static qw_status build_schedule(qw_batch_s* b) {
     if (sa != QW_OK) return sa;
     QW_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<true>, kFusedThreads, b->smem));
   } else {
-    QW_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<false>, kBatchThreads, 0));
+    qw_status sa = smem_attr(batch_kernel<false>, kMarchSmem);
+    if (sa != QW_OK) return sa;
+    QW_CHECK_CUDA(
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<false>, kMarchThreads, kMarchSmem));
   }
   QW_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
   b->grid = std::max(1, per_sm * nsm);
@@ -787,7 +845,7 @@ static qw_status launch_batch(qw_batch_s* b, cudaStream_t s) {
                                                                b->ngroups, b->d_tiles, b->d_rounds, b->total_items,
                                                                b->d_done, b->d_ctl, b->dbg);
   else
-    batch_kernel<false><<<b->grid, kBatchThreads, 0, s>>>(b->d_walks, b->d_groups, b->d_group_item0, b->ngroups,
+    batch_kernel<false><<<b->grid, kMarchThreads, b->smem, s>>>(b->d_walks, b->d_groups, b->d_group_item0, b->ngroups,
                                                           b->d_tiles, b->d_rounds, b->total_items, b->d_done,
                                                           b->d_ctl, b->dbg);
   QW_CHECK_LAUNCH("batch kernel launch");

@@ -36,8 +36,8 @@ const Strip2 kStrips[] = {QW_STRIPS2(X)};
 March2 geometry2(int64_t N, const Strip2& s, int sms, double* us) {
   March2 p{};
   p.N = (int)N;
-  p.tx = 32 * s.kx - 2 * s.t;
-  p.ntx = (p.N + p.tx - 1) / p.tx;
+  const int tx = 32 * s.kx - 2 * s.t;
+  p.ntx = (p.N + tx - 1) / tx;
   const int full = sms * s.ctas * s.nw;  // resident warps
   const int base = std::max(1, full / p.ntx);
   double best = -1.0;

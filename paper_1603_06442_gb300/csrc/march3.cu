@@ -48,14 +48,9 @@ const Tile3 kTiles128[] = {QW_TILES3_C128(X)
 template <typename C> March3<C> geometry3(const Geometry& g, const Tile3& s, int sms, int* grid) {
   March3<C> p{};
   const int M = (int)g.nx;
-  p.M = M;
-  p.perx = M <= 32 * s.kx && M % s.kx == 0;
-  p.lanes = p.perx ? M / s.kx : 32;
-  p.pery = s.nw * s.ky == M;
-  p.tx = p.perx ? M : 32 * s.kx - s.t;
-  p.ty = p.pery ? M : s.nw * s.ky - s.t;
-  p.ntx = (M + p.tx - 1) / p.tx;
-  p.nty = (M + p.ty - 1) / p.ty;
+  p.g = tile3_geo(M, s.kx, s.ky, s.t, s.nw);
+  p.ntx = (M + p.g.tx - 1) / p.g.tx;
+  p.nty = (M + p.g.ty - 1) / p.g.ty;
   *grid = march3_split(p, s.t, sms * s.ctas);
   return p;
 }
@@ -63,7 +58,7 @@ template <typename C> March3<C> geometry3(const Geometry& g, const Tile3& s, int
 double estimate3(const Geometry& g, const Tile3& s, int sms) {
   int grid;
   const March3<float2> p = geometry3<float2>(g, s, sms, &grid);
-  const int P = 2 * p.M;
+  const int P = 2 * p.g.M;
   int iters = p.rounds * (P + 2 * s.t);
   if (p.rest) iters += (p.planes < P ? p.planes : P) + 2 * s.t;
   return 2.5 + iters * s.us;  // us a launch: start and end, and the half-layers of the longest CTA

@@ -125,13 +125,16 @@ template <int N> __device__ __forceinline__ void cp_async_wait() {
 // warp's rows, from the neighbouring warp through shared memory (one barrier per level).
 // A tile is computed with the halo of its T steps (T physical sites per side), or, where the
 // warp's cells (the CTA's rows) are exactly a period of the box, cyclically without one.
+struct Tile3Geo {
+  int M;           // cells per axis
+  int perx, pery;  // cyclic tile along x / y
+  int lanes;       // lanes in use (cyclic x tiles: M / KX, else 32)
+  int tx, ty;      // cells a tile writes along x / y
+};
 template <typename C> struct March3 {
   const C* in[2][4];  // component planes of each coset
   C* out[2][4];
-  int M;              // cells per axis
-  int perx, pery;     // cyclic tile along x / y
-  int lanes;          // lanes in use (cyclic x tiles: M / KX, else 32)
-  int tx, ty;         // cells a tile writes along x / y
+  Tile3Geo g;
   int ntx, nty;       // tiles
   // Which CTA marches which half-layers (march3_split): first `rounds` whole tiles per CTA; of the
   // `rest` tiles left, `per` CTAs each take `planes` half-layers per tile, and the CTAs beyond
@@ -288,19 +291,31 @@ template <typename R, int KX, int KY, int NW> constexpr int march3_smem() {
   return (int)sizeof(typename CplxOf<R>::T) * (kMarch3Stages * 4 * KX * KY * 32 * NW + 2 * 2 * KX * 32 * NW);
 }
 
+// The tile of NW warps of KX cells per lane and KY rows, T steps, on a box of M cells per axis.
+__host__ __device__ inline Tile3Geo tile3_geo(int M, int kx, int ky, int t, int nw) {
+  Tile3Geo g;
+  g.M = M;
+  g.perx = M <= 32 * kx && M % kx == 0;
+  g.lanes = g.perx ? M / kx : 32;
+  g.pery = nw * ky == M;
+  g.tx = g.perx ? M : 32 * kx - t;
+  g.ty = g.pery ? M : nw * ky - t;
+  return g;
+}
+
 // Fill the split of p over `ctas` resident CTAs; returns the grid.  All CTAs walk whole tiles, or
 // equal parts of them, at the same height, so that the halo a tile shares with its neighbours is
 // read while it is in L2; only the CTAs that do not divide evenly take the tiles' ends.
 template <typename C> inline int march3_split(March3<C>& p, int T, int ctas) {
-  const int P = 2 * p.M, nt = p.ntx * p.nty;
+  const int P = 2 * p.g.M, nt = p.ntx * p.nty;
   p.rounds = nt / ctas;
   p.rest = nt - p.rounds * ctas;
   p.per = p.planes = p.extra = 0;
   if (p.rest == 0) return ctas;
-  p.per = ctas / p.rest < p.M ? ctas / p.rest : p.M;
-  p.planes = 2 * ((p.M + p.per - 1) / p.per);
+  p.per = ctas / p.rest < p.g.M ? ctas / p.rest : p.g.M;
+  p.planes = 2 * ((p.g.M + p.per - 1) / p.per);
   const int help = ctas - p.rest * p.per;
-  if (help > 0 && p.per < p.M) {
+  if (help > 0 && p.per < p.g.M) {
     // the longest even part of the main CTAs for which the helpers' load is no longer than theirs
     const int segs = (p.rest + help - 1) / help;
     for (int m = 2; m <= p.planes; m += 2) {
@@ -317,28 +332,91 @@ template <typename C> inline int march3_split(March3<C>& p, int T, int ctas) {
   return p.rounds > 0 ? ctas : p.rest * p.per;
 }
 
-template <typename R, int KX, int KY, int T, int NW, int CTAS>
-__global__ void __launch_bounds__(32 * NW, CTAS)
-    march3d_kernel(const __grid_constant__ March3<typename CplxOf<R>::T> p, const typename CoefOf<R>::T coef) {
+// Half-layers [ls, le) (ls even) of tile (itx, ity), T steps on from the field whose component q of
+// coset c starts at in(c, q), to out(c, q).  All NW warps of the CTA; march_smem as march3_smem says.
+// A component plane of a coset has M^3 < 2^32 cells (a field beyond that would not fit the device),
+// so 32-bit indices on top of the planes' addresses: one instruction a load.
+template <typename R, int KX, int KY, int T, int NW, bool EXACT, typename IN, typename OUT, typename CF>
+__device__ __forceinline__ void march3_segment(const Tile3Geo& g, int itx, int ity, int ls, int le,
+                                               unsigned char* march_smem, IN in, OUT out, const CF& cf) {
   using C = typename CplxOf<R>::T;
   using H = typename HeldOf<R>::T;
   constexpr int NT = 32 * NW, SLOT = 4 * KX * KY * NT;  // threads, values of one staged half-layer
-  extern __shared__ __align__(16) unsigned char march_smem[];
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   C* const stage = reinterpret_cast<C*>(march_smem) + tid;  // [stage][q][ky][kx][thread]
   C* const xch = reinterpret_cast<C*>(march_smem) + kMarch3Stages * SLOT;
-  const auto cf = spread(coef);
-
-  const int M = p.M, P = 2 * M;
+  const int M = g.M, P = 2 * M;
   const unsigned layer = (unsigned)M * M, zend = (unsigned)M * layer;
-  // first cell of a tile's box: a halo of lo0 cells (coset 0) before the first written cell
-  constexpr int lo0 = (T + 1) / 2, lo1 = T / 2;
-  const int sup = p.perx ? (lane == 0 ? p.lanes - 1 : lane - 1) : max(lane - 1, 0);
-  const int sdn = p.perx ? (lane == p.lanes - 1 ? 0 : lane + 1) : min(lane + 1, 31);
+  const int sup = g.perx ? (lane == 0 ? g.lanes - 1 : lane - 1) : max(lane - 1, 0);
+  const int sdn = g.perx ? (lane == g.lanes - 1 ? 0 : lane + 1) : min(lane + 1, 31);
   const int wup = w == 0 ? NW - 1 : w - 1, wdn = w == NW - 1 ? 0 : w + 1;
+  // first cell of the tile's box: a halo of lo0 cells (coset 0) before the first written cell
+  constexpr int lo0 = (T + 1) / 2, lo1 = T / 2;
+  const int xb = g.perx ? 0 : itx * g.tx - lo0, yb = g.pery ? 0 : ity * g.ty - lo0;
+  const int iters = le - ls + 2 * T;
 
-  // Every value of a level that reaches an output is written in the 2 T iterations before it, so
-  // the levels are set once, not per segment.
+  // cell indices in a layer, and which of them are written (bit per cell, by coset) and, with EXACT,
+  // read: not those past what a short last tile needs, which another CTA may be writing (their values
+  // reach no output)
+  const int mx = g.perx ? M - 1 : min(g.tx, M - itx * g.tx) + T - 1;
+  const int my = g.pery ? M - 1 : min(g.ty, M - ity * g.ty) + T - 1;
+  unsigned off[KY][KX], rd = 0u, wr[2] = {0u, 0u}, wrow[2] = {0u, 0u};
+#pragma unroll
+  for (int y = 0; y < KY; ++y) {
+    const int ly = w * KY + y;
+    int gy = (yb + ly) % M;
+    if (gy < 0) gy += M;
+#pragma unroll
+    for (int k = 0; k < KX; ++k) {
+      const int lx = lane * KX + k;
+      int gx = (xb + lx) % M;
+      if (gx < 0) gx += M;
+      off[y][k] = (unsigned)gy * M + gx;
+      if (EXACT && lx <= mx && ly <= my) rd |= 1u << (y * KX + k);
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const int lo = c == 0 ? lo0 : lo1;
+        const bool okx = g.perx ? lx < M : (lx >= lo && lx - lo < g.tx && itx * g.tx + lx - lo < M);
+        const bool oky = g.pery ? ly < M : (ly >= lo && ly - lo < g.ty && ity * g.ty + ly - lo < M);
+        if (okx && oky) wr[c] |= 1u << (y * KX + k);
+        if (oky) wrow[c] |= 1u << y;
+      }
+    }
+  }
+
+  // half-layer ls - T + i is iteration i's arrival; its coset is that of T + i (ls is even)
+  int lin = (ls - T) % P;
+  if (lin < 0) lin += P;
+  unsigned zin = (unsigned)(lin >> 1) * layer;  // first index of its layer
+  int left = iters;
+  // load the next half-layer, of coset CI, into slot
+  auto issue = [&](auto coset, int slot) {
+    constexpr int CI = decltype(coset)::value;
+    if (left > 0) {
+      C* d = stage + slot * SLOT;
+#pragma unroll
+      for (int y = 0; y < KY; ++y)
+#pragma unroll
+        for (int k = 0; k < KX; ++k)
+          if (!EXACT || (rd >> (y * KX + k) & 1u)) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) cp_async_c(d + ((q * KY + y) * KX + k) * NT, in(CI, q) + (zin + off[y][k]));
+          }
+      if (CI == 1) {
+        zin += layer;
+        if (zin == zend) zin = 0;
+      }
+    }
+    --left;
+    cp_async_commit();
+  };
+  using Even = std::integral_constant<int, T & 1>;  // coset of iterations 0, 2, ...
+  using Odd = std::integral_constant<int, (T + 1) & 1>;
+  issue(Even(), 0);
+  issue(Odd(), 1);
+  issue(Even(), 2);
+  static_assert(kMarch3Stages == 4, "three half-layers ahead");
+
   Level3<R, KX, KY> L[T];
 #pragma unroll
   for (int t = 0; t < T; ++t)
@@ -351,6 +429,51 @@ __global__ void __launch_bounds__(32 * NW, CTAS)
         for (int q = 0; q < 4; ++q) L[t].own[y][k][q] = held<0>(C{0, 0});
       }
 
+  unsigned zout = (unsigned)(ls >> 1) * layer;  // layer being written
+  int pair = 0;                                 // slots 0, 1 or 2, 3 hold this pair of arrivals
+  for (int j = 0; j < iters; j += 2) {
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      if (u == 0)
+        issue(Odd(), (pair ^ 2) + 1);
+      else
+        issue(Even(), pair);
+      cp_async_wait<kMarch3Stages - 1>();
+      const unsigned rows = j >= 2 * T ? wrow[u] : 0u;
+      H v[KY][KX][4];
+      const C* s = stage + (pair + u) * SLOT;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+#pragma unroll
+        for (int y = 0; y < KY; ++y)
+#pragma unroll
+          for (int k = 0; k < KX; ++k) v[y][k][q] = held<0>(s[((q * KY + y) * KX + k) * NT]);
+      if (u == 0)
+        march3_levels<0, T, (T & 1), 0>(L, v, xch, 2 * KX * NT, lane, w, wup, wdn, rows, sup, sdn, cf);
+      else
+        march3_levels<0, T, ((T + 1) & 1), 1>(L, v, xch, 2 * KX * NT, lane, w, wup, wdn, rows, sup, sdn, cf);
+      if (j >= 2 * T) {  // half-layer ls + j + u - 2 T: coset u
+#pragma unroll
+        for (int y = 0; y < KY; ++y)
+#pragma unroll
+          for (int k = 0; k < KX; ++k)
+            if (wr[u] >> (y * KX + k) & 1u) {
+#pragma unroll
+              for (int q = 0; q < 4; ++q) out(u, q)[zout + off[y][k]] = value<(T & 1)>(v[y][k][q]);
+            }
+        if (u == 1) zout += layer;
+      }
+    }
+    pair ^= 2;
+  }
+}
+
+template <typename R, int KX, int KY, int T, int NW, int CTAS>
+__global__ void __launch_bounds__(32 * NW, CTAS)
+    march3d_kernel(const __grid_constant__ March3<typename CplxOf<R>::T> p, const typename CoefOf<R>::T coef) {
+  extern __shared__ __align__(16) unsigned char march_smem[];
+  const auto cf = spread(coef);
+  const int P = 2 * p.g.M;
   grid_wait();
   // the CTA's segments [ls, le) of a tile
   const int main_ctas = p.rest * p.per, b = blockIdx.x, tail = P - p.per * p.planes;
@@ -376,104 +499,9 @@ __global__ void __launch_bounds__(32 * NW, CTAS)
       le = (int)min((int64_t)P, ls + (end - pos));
       pos += le - ls;
     }
-    const int itx = tile % p.ntx, ity = tile / p.ntx;
-    const int xb = p.perx ? 0 : itx * p.tx - lo0, yb = p.pery ? 0 : ity * p.ty - lo0;
-    const int iters = le - ls + 2 * T;
-
-    // cell indices in a layer, and which of them are written (bit per cell, by coset).  A component
-    // plane of a coset has M^3 < 2^32 cells (a field beyond that would not fit the device), so
-    // 32-bit indices on top of the planes' addresses in the parameters: one instruction a load.
-    unsigned off[KY][KX], wr[2] = {0u, 0u}, wrow[2] = {0u, 0u};
-#pragma unroll
-    for (int y = 0; y < KY; ++y) {
-      const int ly = w * KY + y;
-      int gy = (yb + ly) % M;
-      if (gy < 0) gy += M;
-#pragma unroll
-      for (int k = 0; k < KX; ++k) {
-        const int lx = lane * KX + k;
-        int gx = (xb + lx) % M;
-        if (gx < 0) gx += M;
-        off[y][k] = (unsigned)gy * M + gx;
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const int lo = c == 0 ? lo0 : lo1;
-          const bool okx = p.perx ? lx < M : (lx >= lo && lx - lo < p.tx && itx * p.tx + lx - lo < M);
-          const bool oky = p.pery ? ly < M : (ly >= lo && ly - lo < p.ty && ity * p.ty + ly - lo < M);
-          if (okx && oky) wr[c] |= 1u << (y * KX + k);
-          if (oky) wrow[c] |= 1u << y;
-        }
-      }
-    }
-
-    // half-layer ls - T + i is iteration i's arrival; its coset is that of T + i (ls is even)
-    int lin = (ls - T) % P;
-    if (lin < 0) lin += P;
-    unsigned zin = (unsigned)(lin >> 1) * layer;  // first index of its layer
-    int left = iters;
-    // load the next half-layer, of coset CI, into slot
-    auto issue = [&](auto coset, int slot) {
-      constexpr int CI = decltype(coset)::value;
-      if (left > 0) {
-        C* d = stage + slot * SLOT;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int y = 0; y < KY; ++y)
-#pragma unroll
-            for (int k = 0; k < KX; ++k) cp_async_c(d + ((q * KY + y) * KX + k) * NT, p.in[CI][q] + (zin + off[y][k]));
-        if (CI == 1) {
-          zin += layer;
-          if (zin == zend) zin = 0;
-        }
-      }
-      --left;
-      cp_async_commit();
-    };
-    using Even = std::integral_constant<int, T & 1>;  // coset of iterations 0, 2, ...
-    using Odd = std::integral_constant<int, (T + 1) & 1>;
-    issue(Even(), 0);
-    issue(Odd(), 1);
-    issue(Even(), 2);
-    static_assert(kMarch3Stages == 4, "three half-layers ahead");
-
-    unsigned zout = (unsigned)(ls >> 1) * layer;  // layer being written
-    int pair = 0;                                 // slots 0, 1 or 2, 3 hold this pair of arrivals
-    for (int j = 0; j < iters; j += 2) {
-#pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        if (u == 0)
-          issue(Odd(), (pair ^ 2) + 1);
-        else
-          issue(Even(), pair);
-        cp_async_wait<kMarch3Stages - 1>();
-        const unsigned rows = j >= 2 * T ? wrow[u] : 0u;
-        H v[KY][KX][4];
-        const C* s = stage + (pair + u) * SLOT;
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int y = 0; y < KY; ++y)
-#pragma unroll
-            for (int k = 0; k < KX; ++k) v[y][k][q] = held<0>(s[((q * KY + y) * KX + k) * NT]);
-        if (u == 0)
-          march3_levels<0, T, (T & 1), 0>(L, v, xch, 2 * KX * NT, lane, w, wup, wdn, rows, sup, sdn, cf);
-        else
-          march3_levels<0, T, ((T + 1) & 1), 1>(L, v, xch, 2 * KX * NT, lane, w, wup, wdn, rows, sup, sdn, cf);
-        if (j >= 2 * T) {  // half-layer ls + j + u - 2 T: coset u
-#pragma unroll
-          for (int y = 0; y < KY; ++y)
-#pragma unroll
-            for (int k = 0; k < KX; ++k)
-              if (wr[u] >> (y * KX + k) & 1u) {
-#pragma unroll
-                for (int q = 0; q < 4; ++q) p.out[u][q][zout + off[y][k]] = value<(T & 1)>(v[y][k][q]);
-              }
-          if (u == 1) zout += layer;
-        }
-      }
-      pair ^= 2;
-    }
+    march3_segment<R, KX, KY, T, NW, false>(
+        p.g, tile % p.ntx, tile / p.ntx, ls, le, march_smem, [&](int c, int q) { return p.in[c][q]; },
+        [&](int c, int q) { return p.out[c][q]; }, cf);
   }
 }
 

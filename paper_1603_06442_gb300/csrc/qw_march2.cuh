@@ -17,7 +17,7 @@ struct March2 {
   const float2* in[4];
   float2* out[4];
   int N;
-  int tx, ntx;  // columns a strip writes, strips
+  int ntx;      // strips (of 32 KX - 2 T written columns)
   int rows;     // rows a warp writes
   int chunks;   // chunks of rows per strip
 };
@@ -77,37 +77,35 @@ constexpr int kMarch2Stages = 4;  // rows in flight per warp
 
 template <int KX, int NW> constexpr int march2_smem() { return 8 * kMarch2Stages * 4 * KX * 32 * NW; }
 
-template <int KX, int T, int NW, int CTAS>
-__global__ void __launch_bounds__(32 * NW, CTAS) march2d_kernel(const __grid_constant__ March2 p, const Coef32 coef) {
-  constexpr int NT = 32 * NW, SLOT = 4 * KX * NT;
-  extern __shared__ __align__(16) unsigned char march_smem[];
+// Rows [ys, ye) of a strip by one warp (w of NW in the CTA), T steps on from the field whose component q
+// starts at in(q), to out(q).  A component plane has N^2 < 2^32 sites: 32-bit indices.
+template <int KX, int T, int NW, bool EXACT, typename IN, typename OUT>
+__device__ __forceinline__ void march2_rows(int N, int strip, int ys, int ye, unsigned char* march_smem, IN in, OUT out,
+                                            const CoefF2& cf) {
+  constexpr int NT = 32 * NW, SLOT = 4 * KX * NT, TX = 32 * KX - 2 * T;
   const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
   // [stage][q][warp][column]: a row's columns are fetched 32 apart (whole sectors) and read KX
   // neighbours at a time
   float2* const stage = reinterpret_cast<float2*>(march_smem) + w * (32 * KX);
-  const CoefF2 cf = spread(coef);
-  const int N = p.N;
-  grid_wait();
-  const int64_t item = (int64_t)blockIdx.x * NW + w;
-  if (item >= (int64_t)p.ntx * p.chunks) return;  // whole warps: nothing below meets another warp
-  const int strip = (int)(item % p.ntx), chunk = (int)(item / p.ntx);
-  const int ys = chunk * p.rows, ye = min(ys + p.rows, N);
   const int iters = ye - ys + 2 * T;
   const int up = max(lane - 1, 0), dn = min(lane + 1, 31);
 
-  unsigned fetch[KX], off[KX], wr = 0u;  // the columns the lane fetches, and those it owns
+  // the columns the lane fetches (with EXACT, none past those a short last strip needs, which another
+  // warp may be writing: their values reach no output), and those it owns
+  const int mx = min(TX, N - strip * TX) + T - 1;
+  unsigned fetch[KX], off[KX], rd = 0u, wr = 0u;
 #pragma unroll
   for (int k = 0; k < KX; ++k) {
-    int fx = (strip * p.tx + k * 32 + lane - T) % N;
+    int fx = (strip * TX + k * 32 + lane - T) % N;
     if (fx < 0) fx += N;
     fetch[k] = fx;
+    if (EXACT && k * 32 + lane - T <= mx) rd |= 1u << k;
     const int lx = lane * KX + k - T;  // column relative to the strip's first written one
-    int gx = (strip * p.tx + lx) % N;
+    int gx = (strip * TX + lx) % N;
     if (gx < 0) gx += N;
     off[k] = gx;
-    if (lx >= 0 && lx < p.tx && strip * p.tx + lx < N) wr |= 1u << k;
+    if (lx >= 0 && lx < TX && strip * TX + lx < N) wr |= 1u << k;
   }
-  // a component plane has N^2 < 2^32 sites (march_supported): 32-bit indices
   int rin = (ys - T) % N;
   if (rin < 0) rin += N;
   unsigned yin = (unsigned)rin * N;
@@ -117,9 +115,11 @@ __global__ void __launch_bounds__(32 * NW, CTAS) march2d_kernel(const __grid_con
     if (left > 0) {
       float2* d = stage + slot * SLOT;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+      for (int k = 0; k < KX; ++k)
+        if (!EXACT || (rd >> k & 1u)) {
 #pragma unroll
-        for (int k = 0; k < KX; ++k) cp_async_c(d + q * KX * NT + k * 32 + lane, p.in[q] + (yin + fetch[k]));
+          for (int q = 0; q < 4; ++q) cp_async_c(d + q * KX * NT + k * 32 + lane, in(q) + (yin + fetch[k]));
+        }
       yin += N;
       if (yin == yend) yin = 0;
     }
@@ -166,13 +166,26 @@ __global__ void __launch_bounds__(32 * NW, CTAS) march2d_kernel(const __grid_con
         for (int k = 0; k < KX; ++k)
           if (wr >> k & 1u) {
 #pragma unroll
-            for (int q = 0; q < 4; ++q) p.out[q][yout + off[k]] = value<(T & 1)>(v[k][q]);
+            for (int q = 0; q < 4; ++q) out(q)[yout + off[k]] = value<(T & 1)>(v[k][q]);
           }
         yout += N;
       }
     }
     slot ^= 2;
   }
+}
+
+template <int KX, int T, int NW, int CTAS>
+__global__ void __launch_bounds__(32 * NW, CTAS) march2d_kernel(const __grid_constant__ March2 p, const Coef32 coef) {
+  extern __shared__ __align__(16) unsigned char march_smem[];
+  const CoefF2 cf = spread(coef);
+  grid_wait();
+  const int64_t item = (int64_t)blockIdx.x * NW + (threadIdx.x >> 5);
+  if (item >= (int64_t)p.ntx * p.chunks) return;  // whole warps: nothing below meets another warp
+  const int ys = (int)(item / p.ntx) * p.rows;
+  march2_rows<KX, T, NW, false>(
+      p.N, (int)(item % p.ntx), ys, min(ys + p.rows, p.N), march_smem, [&](int q) { return p.in[q]; },
+      [&](int q) { return p.out[q]; }, cf);
 }
 
 }  // namespace qw

@@ -72,3 +72,20 @@ def test_marching_matches_the_oracle(qb, dtype, dim, N):
     exp = walk.to_device(dim, N, walk.step(dim, m, walk.from_device(dim, N, a), t))
     err = np.linalg.norm(x.cpu().numpy() - exp) / np.linalg.norm(exp)
     assert err <= (1e-5 if dtype == "c64" else 1e-11)
+
+
+def test_batch_rounds_equal_plain_bit_for_bit(qb):
+    """A batch's default rounds (marching tiles of every walk in one launch): walks around the tiles'
+    sizes, step counts with every remainder."""
+    spec = [(d, N, 0.05 * (i % 9), 5 + i) for i, (d, N) in enumerate(SIZES) if d > 1] + [(1, 300, 0.2, 9)]
+    fields = [field(d, N, "c64") for d, N, m, t in spec]
+    batch = qb.Batch([(d, N, m, t, x) for (d, N, m, t), x in zip(spec, fields)])
+    batch.run()
+    batch.sync()
+    batch.close()
+    for (d, N, m, t), got in zip(spec, fields):
+        plan = qb.Plan(d, N, m, "c64")
+        want = field(d, N, "c64")
+        plan.step(want, t)
+        plan.close()
+        assert torch.equal(got, want), (d, N, t)
