@@ -174,8 +174,10 @@ __global__ void __launch_bounds__(256) fft_pass_kernel(typename Cx<T>::t* __rest
 
 // MOM (forward strided passes of the observables): the position moments of the loaded lines
 // (FftMoments) are summed before the transform, one partial per CTA.
-template <typename T, bool INV, int R1, int R2, bool CONTIG, bool MOM = false>
-__global__ void __launch_bounds__(256) fft2f_kernel(typename Cx<T>::t* data, const typename Cx<T>::t* src, FftPass p,
+// NT: threads per CTA (256, or 128 for FP64 lines too few to fill the SMs: an FP64 instruction holds a
+// quarter of an SM for 64 clocks a warp, so four warps an SM finish in half the time of eight).
+template <typename T, bool INV, int R1, int R2, bool CONTIG, bool MOM = false, int NT = 256>
+__global__ void __launch_bounds__(NT) fft2f_kernel(typename Cx<T>::t* data, const typename Cx<T>::t* src, FftPass p,
                                                     const typename Cx<T>::t* __restrict__ tw_line,
                                                     const typename Cx<T>::t* __restrict__ tw_hi,
                                                     const typename Cx<T>::t* __restrict__ tw_lo,
@@ -183,11 +185,12 @@ __global__ void __launch_bounds__(256) fft2f_kernel(typename Cx<T>::t* data, con
   using V = typename Cx<T>::t;
   constexpr int L = R1 * R2;
   constexpr int TPL = R1 > R2 ? R1 : R2;  // threads per line
-  constexpr int C = 256 / TPL;            // lines per CTA (C * TPL <= 256 threads work)
+  constexpr int C = NT / TPL;             // lines per CTA (C * TPL <= NT threads work)
   constexpr int CP = (C % 2 == 0) ? C + 1 : C;  // odd line-minor pitch
   extern __shared__ __align__(16) unsigned char f2_smem[];
   V* sm = reinterpret_cast<V*>(f2_smem);
   const int tid = threadIdx.x;
+  grid_wait();
   const int64_t S = p.S;
   const int64_t nlines = p.O * S;
   const int64_t l0 = (int64_t)blockIdx.x * C;
@@ -206,19 +209,19 @@ __global__ void __launch_bounds__(256) fft2f_kernel(typename Cx<T>::t* data, con
   // copies go straight to shared memory, so all of them are in flight at once without
   // holding registers (zero-filled past the last line)
   if (CONTIG) {  // S == 1: the CTA's lines are one contiguous run (never a twiddled pass)
-    // element e = tid + 256 j of the run sits at line e / L, position e % L; both come
+    // element e = tid + NT j of the run sits at line e / L, position e % L; both come
     // from tid / L and tid % L plus compile-time offsets (no division per element)
-    constexpr int NE = (C * L + 255) / 256;
+    constexpr int NE = (C * L + NT - 1) / NT;
     const int t_c = tid / L, t_x = tid - (tid / L) * L;
 #pragma unroll
     for (int j = 0; j < NE; ++j) {
-      int xx = t_x + (256 * j) % L, cc = t_c + (256 * j) / L;
+      int xx = t_x + (NT * j) % L, cc = t_c + (NT * j) / L;
       if (xx >= L) {
         xx -= L;
         ++cc;
       }
       const bool ok = l0 + cc < nlines;
-      if (cc < C) cp_async_elem(&sm[cc + CP * xx], ok ? src + l0 * L + tid + 256 * j : src, ok);
+      if (cc < C) cp_async_elem(&sm[cc + CP * xx], ok ? src + l0 * L + tid + NT * j : src, ok);
     }
     cp_async_wait_all();
   } else if (r < TPL) {
@@ -292,16 +295,16 @@ __global__ void __launch_bounds__(256) fft2f_kernel(typename Cx<T>::t* data, con
   }
   // ---- store
   if (CONTIG) {
-    constexpr int NE = (C * L + 255) / 256;
+    constexpr int NE = (C * L + NT - 1) / NT;
     const int t_c = tid / L, t_x = tid - (tid / L) * L;
 #pragma unroll
     for (int j = 0; j < NE; ++j) {
-      int xx = t_x + (256 * j) % L, cc = t_c + (256 * j) / L;
+      int xx = t_x + (NT * j) % L, cc = t_c + (NT * j) / L;
       if (xx >= L) {
         xx -= L;
         ++cc;
       }
-      if (cc < C && l0 + cc < nlines) data[l0 * L + tid + 256 * j] = sm[cc + CP * xx];
+      if (cc < C && l0 + cc < nlines) data[l0 * L + tid + NT * j] = sm[cc + CP * xx];
     }
   } else if (r < TPL) {
 #pragma unroll 4
@@ -314,10 +317,10 @@ __global__ void __launch_bounds__(256) fft2f_kernel(typename Cx<T>::t* data, con
   }
 }
 
-template <typename T, bool INV, int R1, int R2>
-static qw_status launch_2f(const FftPass& p, void* data, const void* src, cudaStream_t st) {
+template <typename T, bool INV, int R1, int R2, int NT>
+static qw_status launch_2f_nt(const FftPass& p, void* data, const void* src, bool overlap, cudaStream_t st) {
   using V = typename Cx<T>::t;
-  constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = 256 / TPL;
+  constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = NT / TPL;
   const size_t smem = (size_t)L * ((C % 2 == 0) ? C + 1 : C) * sizeof(V);
   const int64_t nlines = p.O * p.S;
   const int64_t grid = (nlines + C - 1) / C;
@@ -325,21 +328,22 @@ static qw_status launch_2f(const FftPass& p, void* data, const void* src, cudaSt
     set_error("FFT grid too large");
     return QW_EINVAL;
   }
-  if (p.S == 1) {
-    const qw_status sa = smem_attr(fft2f_kernel<T, INV, R1, R2, true>, (int)smem);
-    if (sa != QW_OK) return sa;
-    fft2f_kernel<T, INV, R1, R2, true><<<(unsigned)grid, 256, smem, st>>>(
-        static_cast<V*>(data), static_cast<const V*>(src), p, static_cast<const V*>(p.tw_line), static_cast<const V*>(p.tw_hi),
-        static_cast<const V*>(p.tw_lo));
-  } else {
-    const qw_status sa = smem_attr(fft2f_kernel<T, INV, R1, R2, false>, (int)smem);
-    if (sa != QW_OK) return sa;
-    fft2f_kernel<T, INV, R1, R2, false><<<(unsigned)grid, 256, smem, st>>>(
-        static_cast<V*>(data), static_cast<const V*>(src), p, static_cast<const V*>(p.tw_line), static_cast<const V*>(p.tw_hi),
-        static_cast<const V*>(p.tw_lo));
-  }
-  QW_CHECK_LAUNCH("fft two-factor pass launch");
-  return QW_OK;
+  auto* kernel = p.S == 1 ? fft2f_kernel<T, INV, R1, R2, true, false, NT> : fft2f_kernel<T, INV, R1, R2, false, false, NT>;
+  const qw_status sa = smem_attr(kernel, (int)smem);
+  if (sa != QW_OK) return sa;
+  return launch_overlapped(kernel, (unsigned)grid, NT, (int)smem, overlap, st, static_cast<V*>(data),
+                           static_cast<const V*>(src), p, static_cast<const V*>(p.tw_line),
+                           static_cast<const V*>(p.tw_hi), static_cast<const V*>(p.tw_lo), FftMoments{});
+}
+
+template <typename T, bool INV, int R1, int R2>
+static qw_status launch_2f(const FftPass& p, void* data, const void* src, cudaStream_t st) {
+  constexpr int TPL = R1 > R2 ? R1 : R2;
+  const int64_t nlines = p.O * p.S;
+  const bool overlap = nlines * p.L * (int64_t)sizeof(typename Cx<T>::t) <= (4 << 20);  // as small_field
+  if constexpr (sizeof(T) == 8)
+    if (nlines <= 152 * (256 / TPL)) return launch_2f_nt<T, INV, R1, R2, 128>(p, data, src, overlap, st);
+  return launch_2f_nt<T, INV, R1, R2, 256>(p, data, src, overlap, st);
 }
 
 // f(R1, R2) (as integral constants) for a register length L >= 64; false for other lengths.

@@ -117,6 +117,10 @@ struct Geometry {
 
 bool make_geometry(int dim, int64_t N, Geometry* g);
 
+// Fields whose kernels run a few us each: their passes are launched to overlap (launch_overlapped;
+// the split of L1 and shared memory does not matter where most of an SM is idle).
+inline bool small_field(const Geometry& g, qw_dtype dt) { return g.elems * (dt == QW_C64 ? 8 : 16) <= (4 << 20); }
+
 // Fields need only element alignment (8 bytes in complex64); kernels that move 16-byte
 // vectors are chosen only for fields that are 16-byte aligned.
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }

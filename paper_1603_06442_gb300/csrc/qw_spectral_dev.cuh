@@ -185,10 +185,24 @@ __device__ __forceinline__ void coset_phase(int64_t fsum, int64_t M, T& ar, T& a
 
 // Position of the thread in a 3D launch over (nx, ny, nz); false when outside.
 __device__ __forceinline__ bool grid_pos(const AxesDev& a, int64_t& x, int64_t& y, int64_t& z) {
-  x = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  y = blockIdx.y;
-  z = blockIdx.z;
-  return x < a.len[0];
+  // one thread per position of the box, x fastest: a grid over rows would leave most of a CTA idle
+  // on boxes narrower than it (a box of 81^3 cells used 81 of 256 threads)
+  const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t total = a.len[0] * a.len[1] * a.len[2];
+  if (idx >= total) return false;
+  if (total <= 0x7fffffff) {  // 32-bit index arithmetic
+    const int i = (int)idx, nx = (int)a.len[0], ny = (int)a.len[1];
+    const int yz = i / nx;
+    x = i - yz * nx;
+    z = yz / ny;
+    y = yz - (int)z * ny;
+  } else {
+    x = idx % a.len[0];
+    const int64_t yz = idx / a.len[0];
+    y = yz % a.len[1];
+    z = yz / a.len[1];
+  }
+  return true;
 }
 
 // (cos, sin)(2 pi nu t) for nu = hi + lo (FP32 pair) and integer t < 2^24, in FP32:

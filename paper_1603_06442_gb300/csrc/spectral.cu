@@ -145,6 +145,7 @@ __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t
                                                      const double* __restrict__ norm0,
                                                      typename Cx2<T>::t* __restrict__ data) {
   using V = typename Cx2<T>::t;
+  grid_wait();
   // optional normalisation of the initial state, folded into the 1/|V| scale
   const T scale = norm0 ? (sizeof(T) == 8 ? (T)((double)scale_in / sqrt(norm0[0]))
                                            : (T)(scale_in * rsqrtf((float)norm0[0])))
@@ -366,9 +367,13 @@ __global__ void __launch_bounds__(kFoldThreads) fold2_kernel(const double* __res
 static int64_t kcount(const Geometry& g) { return g.vol; }
 
 
-static dim3 grid3(const Geometry& g) {
-  return dim3((unsigned)((g.nx + 255) / 256), (unsigned)g.ny, (unsigned)g.nz);
+// Threads per CTA and CTAs of a pointwise kernel.  FP64 on a small box: an FP64 instruction holds a
+// quarter of an SM for 64 clocks a warp, so a CTA of one warp per quarter, on as many SMs as there are.
+constexpr int kPointThreads = 256, kPointSmall = 128;
+static int point_threads(const Geometry& g, qw_dtype dt) {
+  return dt == QW_C128 && g.vol <= 152 * kPointThreads ? kPointSmall : kPointThreads;
 }
+static unsigned point_grid(const Geometry& g, int threads) { return (unsigned)((g.vol + threads - 1) / threads); }
 
 // complex128 plans: the double-double omega table (16 bytes per stored wave vector).  The
 // per-axis and anchor tables it needs live in one temporary buffer (synchronous).
@@ -400,7 +405,7 @@ static qw_status launch_omega_table_dd(const Geometry& g, const SpecAxes& ax, do
   }
   dd_table_kernel<<<5, 256, 0, st>>>(anch, 1025, 2048);
   dd_mass_kernel<<<1, 1, 0, st>>>(m, nbox);
-  omega_dd_kernel<<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), m, nbox, tabs[0], tabs[1], tabs[2], anch,
+  omega_dd_kernel<<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), m, nbox, tabs[0], tabs[1], tabs[2], anch,
                                             reinterpret_cast<double2*>(omega));
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
@@ -412,7 +417,7 @@ static qw_status launch_omega_table_dd(const Geometry& g, const SpecAxes& ax, do
 qw_status launch_omega_table(const Geometry& g, const SpecAxes& ax, double n, double m, double* omega,
                               cudaStream_t st, bool split) {
   if (!split) return launch_omega_table_dd(g, ax, m, omega, st);
-  omega_split_kernel<<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), n, m, reinterpret_cast<float2*>(omega));
+  omega_split_kernel<<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), n, m, reinterpret_cast<float2*>(omega));
   QW_CHECK_LAUNCH("omega table launch");
   return QW_OK;
 }
@@ -422,15 +427,14 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
                                   const double* norm0) {
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
+  const int threads = point_threads(g, dt);
+  const bool overlap = small_field(g, dt);
   if (dt == QW_C64)
-    evolve_kernel<float><<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), omega,
-                                                         make_time(t), (float)inv, norm0,
-                                                         static_cast<float2*>(psi_hat));
-  else
-    evolve_kernel<double><<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), omega,
-                                                          make_time(t), inv, norm0, static_cast<double2*>(psi_hat));
-  QW_CHECK_LAUNCH("evolve launch");
-  return QW_OK;
+    return launch_overlapped(evolve_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
+                             count, make_mass(n, m), omega, make_time(t), (float)inv, norm0,
+                             static_cast<float2*>(psi_hat));
+  return launch_overlapped(evolve_kernel<double>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
+                           count, make_mass(n, m), omega, make_time(t), inv, norm0, static_cast<double2*>(psi_hat));
 }
 
 qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m, void* psi_hat,
@@ -438,10 +442,10 @@ qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
   if (dt == QW_C64)
-    fw_kernel<float><<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), (float)inv,
+    fw_kernel<float><<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), (float)inv,
                                                static_cast<float2*>(psi_hat));
   else
-    fw_kernel<double><<<grid3(g), 256, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), inv,
+    fw_kernel<double><<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), inv,
                                                 static_cast<double2*>(psi_hat));
   QW_CHECK_LAUNCH("Foldy-Wouthuysen launch");
   return QW_OK;
