@@ -261,6 +261,9 @@ qw_status launch_weights_fused_x(const Geometry& g, const SpecAxes& ax, const Ff
 // inverse transform's 1/|V| scale folded in).
 qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m, void* psi_hat,
                               cudaStream_t st);
+// The fused x pass with the Foldy-Wouthuysen coefficients in place of D_k^t.
+qw_status launch_fw_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m, void* psi,
+                            cudaStream_t st);
 qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m,
                                   const double* omega, int64_t t, void* psi_hat, cudaStream_t st,
                                   const double* norm0 = nullptr);

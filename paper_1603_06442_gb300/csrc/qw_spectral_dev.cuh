@@ -648,6 +648,117 @@ __device__ __forceinline__ void weights_point(int dim, const AxesDev& a, int64_t
   }
 }
 
+// Foldy-Wouthuysen coefficients of one wave vector (the Remark on the Newton-Wigner
+// position): w_r = u_r(k)^dag v on the paper's eigenvectors of D_k (Eq. evecs-D),
+// r = (s, p) in the order (+,+), (+,-), (-,+), (-,-):
+//   u_{s,p} = (A, -p B e^{i phi}, -s C, s p D) / 2,  A = sqrt((1 - p vW)(1 + s p vD)),
+//   B = sqrt((1 + p vW)(1 + s p vD)), C = sqrt((1 - p vW)(1 - s p vD)), D = sqrt((1 + p vW)(1 - s p vD)),
+// vW = -n~_z / |n~|, e^{i phi} = -(n~_x + i n~_y) / |(n~_x, n~_y)| (phi = Arg(n~_y - i n~_x) - pi/2),
+// vD = n |n~| / sqrt(m^2 + n^2 |n~|^2); vW = 0, phi = 0, vD = 0 where their ratios are 0/0.
+// 1D (the decoupled 2x2 walk): u_+ = (cos th/2, -sin th/2), u_- = (sin th/2, cos th/2),
+// th = atan2(m, n sin k).
+template <typename T, int S>
+__device__ __forceinline__ void fw_apply(T u, T nx, T ny, T nz, T n, T m, typename Cx2<T>::t (&v)[S]) {
+  using V = typename Cx2<T>::t;
+  (void)u;
+  if (S == 2) {
+    const T th = atan2(m, n * nz);
+    const T c = cos((T)0.5 * th), sn = sin((T)0.5 * th);
+    const V a = v[0], b = v[1];
+    v[0].x = c * a.x - sn * b.x;
+    v[0].y = c * a.y - sn * b.y;
+    v[1].x = sn * a.x + c * b.x;
+    v[1].y = sn * a.y + c * b.y;
+    return;
+  }
+  const T tiny = sizeof(T) == 8 ? (T)1e-12 : (T)1e-6;
+  const T r = sqrt(nx * nx + ny * ny + nz * nz);
+  T vW = r < tiny ? (T)0 : -nz / r;
+  vW = vW > (T)1 ? (T)1 : (vW < (T)-1 ? (T)-1 : vW);
+  const T wa = sqrt(nx * nx + ny * ny);
+  const T ec = wa > tiny ? -nx / wa : (T)1, es = wa > tiny ? -ny / wa : (T)0;
+  const T den = sqrt(m * m + n * n * r * r);
+  T vD = den > tiny ? n * r / den : (T)0;
+  vD = vD > (T)1 ? (T)1 : (vD < (T)-1 ? (T)-1 : vD);
+  // e^{-i phi} v1, e^{-i phi} v3
+  V t1, t3;
+  t1.x = ec * v[1].x + es * v[1].y;
+  t1.y = ec * v[1].y - es * v[1].x;
+  t3.x = ec * v[3].x + es * v[3].y;
+  t3.y = ec * v[3].y - es * v[3].x;
+  V w[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const T sg = q < 2 ? (T)1 : (T)-1, pp = (q & 1) ? (T)-1 : (T)1;
+    const T A = (T)0.5 * sqrt(((T)1 - pp * vW) * ((T)1 + sg * pp * vD));
+    const T B = (T)0.5 * sqrt(((T)1 + pp * vW) * ((T)1 + sg * pp * vD));
+    const T C = (T)0.5 * sqrt(((T)1 - pp * vW) * ((T)1 - sg * pp * vD));
+    const T D = (T)0.5 * sqrt(((T)1 + pp * vW) * ((T)1 - sg * pp * vD));
+    w[q].x = A * v[0].x - pp * B * t1.x - sg * C * v[2].x + sg * pp * D * t3.x;
+    w[q].y = A * v[0].y - pp * B * t1.y - sg * C * v[2].y + sg * pp * D * t3.y;
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) v[q] = w[q];
+}
+
+// The Foldy-Wouthuysen coefficients, times the scale, of the spectral values of storage position
+// (x, y, z) (v as in evolve_point).
+template <typename T>
+__device__ __forceinline__ void fw_point(int dim, const AxesDev& a, int64_t x, int64_t y, int64_t z, const Mass& ms,
+                                         T scale, typename Cx2<T>::t (&v)[8]) {
+  using V = typename Cx2<T>::t;
+  const T n = sizeof(T) == 8 ? (T)ms.n : (T)ms.nf, m = sizeof(T) == 8 ? (T)ms.m : (T)ms.mf;
+  int64_t f[3], fs;
+  wave_vectors(dim, x, y, z, a, f, fs);
+  if (dim == 1) {
+    V w[2] = {v[0], v[1]};
+    T u, nx, ny, nz;
+    symbol_tab<T>(1, a, f[0], f[1], f[2], 0, u, nx, ny, nz);
+    fw_apply<T, 2>(u, nx, ny, nz, n, m, w);
+    v[0] = make_vec(w[0], scale);
+    v[1] = make_vec(w[1], scale);
+  } else if (dim == 2) {
+    V w[4] = {v[0], v[1], v[2], v[3]};
+    T u, nx, ny, nz;
+    symbol_tab<T>(2, a, f[0], f[1], f[2], 0, u, nx, ny, nz);
+    fw_apply<T, 4>(u, nx, ny, nz, n, m, w);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = make_vec(w[q], scale);
+  } else {
+    // BCC: the two wave vectors q0, q1 of the cell from the coset mix, as in evolve_point
+    T ar, ai;
+    coset_phase<T>(fs, a.len[0], ar, ai);
+    V c0[4], c1[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      V b;
+      b.x = ar * v[4 + q].x + ai * v[4 + q].y;
+      b.y = ar * v[4 + q].y - ai * v[4 + q].x;
+      c0[q].x = (T)0.5 * (v[q].x + b.x);
+      c0[q].y = (T)0.5 * (v[q].y + b.y);
+      c1[q].x = (T)0.5 * (v[q].x - b.x);
+      c1[q].y = (T)0.5 * (v[q].y - b.y);
+    }
+    T u, nx, ny, nz;
+    symbol_tab<T>(3, a, f[0], f[1], f[2], 0, u, nx, ny, nz);
+    fw_apply<T, 4>(u, nx, ny, nz, n, m, c0);
+    symbol_tab<T>(3, a, f[0], f[1], f[2], 1, u, nx, ny, nz);
+    fw_apply<T, 4>(u, nx, ny, nz, n, m, c1);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      V s0, d, s1;
+      s0.x = c0[q].x + c1[q].x;
+      s0.y = c0[q].y + c1[q].y;
+      d.x = c0[q].x - c1[q].x;
+      d.y = c0[q].y - c1[q].y;
+      s1.x = ar * d.x - ai * d.y;
+      s1.y = ar * d.y + ai * d.x;
+      v[q] = make_vec(s0, scale);
+      v[4 + q] = make_vec(s1, scale);
+    }
+  }
+}
+
 // Byte offset of the row constants after the L x CP line buffer (16-byte aligned).
 __host__ __device__ constexpr size_t fused_rowc_offset(int L, int CP) {
   return (((size_t)L * CP * sizeof(float2)) + 15) & ~size_t(15);
@@ -724,6 +835,72 @@ __device__ __forceinline__ void evolve_bcc_row(const AxesDev& a, int k, float4 r
   }
 }
 
+// 1 / sqrt(x) for x > 0 in FP32 with one Newton step.
+__device__ __forceinline__ float rsqrt_newton(float x) {
+  const float r = rsqrtf(x);
+  return r * fmaf(-0.5f * x * r, r, 1.5f);
+}
+
+// The coefficients of one wave vector from the four products p = sqrt((1 -+ vW)(1 +- vD)) (ae, be, af,
+// bf: a = 1 - vW, b = 1 + vW, e = 1 + vD, f = 1 - vD; every A, B, C, D of fw_apply is one of them).
+__device__ __forceinline__ void fw_row_apply(float ae, float be, float af, float bf, float ec, float es,
+                                             float2 (&v)[4]) {
+  const float2 t1 = make_float2(ec * v[1].x + es * v[1].y, ec * v[1].y - es * v[1].x);  // e^{-i phi} v1, v3
+  const float2 t3 = make_float2(ec * v[3].x + es * v[3].y, ec * v[3].y - es * v[3].x);
+  const float2 w0 = make_float2(ae * v[0].x - be * t1.x - af * v[2].x + bf * t3.x,
+                                ae * v[0].y - be * t1.y - af * v[2].y + bf * t3.y);
+  const float2 w1 = make_float2(bf * v[0].x + af * t1.x - be * v[2].x - ae * t3.x,
+                                bf * v[0].y + af * t1.y - be * v[2].y - ae * t3.y);
+  const float2 w2 = make_float2(af * v[0].x - bf * t1.x + ae * v[2].x - be * t3.x,
+                                af * v[0].y - bf * t1.y + ae * v[2].y - be * t3.y);
+  const float2 w3 = make_float2(be * v[0].x + ae * t1.x + bf * v[2].x + af * t3.x,
+                                be * v[0].y + ae * t1.y + bf * v[2].y + af * t3.y);
+  v[0] = w0;
+  v[1] = w1;
+  v[2] = w2;
+  v[3] = w3;
+}
+
+// fw_point for a BCC cell in complex64 from its row constants rc and x frequency k.  The half
+// spectrum q1 has the opposite n~: vW and e^{i phi} change sign, vD stays (with the 0/0 conventions of
+// fw_apply), so the square roots serve both.
+__device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, float4 rc, const Mass& ms, float scale,
+                                           float2 (&v)[8]) {
+  float cx, sx;
+  tab<float>(a, 0, k, cx, sx);
+  const float nx = sx * rc.x - cx * rc.y, ny = cx * rc.z + sx * rc.w, nz = cx * rc.w - sx * rc.z;
+  const float pr = rc.x - rc.y, pim = rc.w + rc.z;
+  const float ar = cx * pr - sx * pim, ai = cx * pim + sx * pr;  // a = exp(i (k1 + k2 + k3) / 2)
+  const float wa2 = fmaf(nx, nx, ny * ny), r2 = fmaf(nz, nz, wa2);
+  constexpr float tiny2 = 1e-12f;  // (1e-6)^2, as in fw_apply
+  const bool has_w = wa2 > tiny2, has_r = r2 >= tiny2;
+  const float iwa = has_w ? rsqrt_newton(wa2) : 0.f;
+  // correctly rounded: 1 -+ vW and 1 - vD must vanish where n~ lies along z or m = 0 (an error of an
+  // ulp in vW would be one of 2e-4 in its square root)
+  const float r = sqrtf(r2);
+  const float vW = has_r ? fminf(1.f, fmaxf(-1.f, -nz / r)) : 0.f;
+  const float den2 = fmaf(ms.nf * ms.nf, r2, ms.mf * ms.mf);
+  const float vD = den2 > tiny2 ? fminf(1.f, ms.nf * r / sqrtf(den2)) : 0.f;
+  const float pa = 1.f - vW, pb = 1.f + vW, pe = 1.f + vD, pf = 1.f - vD;
+  const float hs = 0.25f * scale;  // the halves of the coset mix and of the eigenvectors
+  const float ae = hs * sqrtf(pa * pe), be = hs * sqrtf(pb * pe), af = hs * sqrtf(pa * pf), bf = hs * sqrtf(pb * pf);
+  float2 c0[4], c1[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float bx = ar * v[4 + q].x + ai * v[4 + q].y, by = ar * v[4 + q].y - ai * v[4 + q].x;
+    c0[q] = make_float2(v[q].x + bx, v[q].y + by);
+    c1[q] = make_float2(v[q].x - bx, v[q].y - by);
+  }
+  fw_row_apply(ae, be, af, bf, has_w ? -nx * iwa : 1.f, -ny * iwa, c0);
+  fw_row_apply(be, ae, bf, af, has_w ? nx * iwa : 1.f, ny * iwa, c1);
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    const float dx = c0[q].x - c1[q].x, dy = c0[q].y - c1[q].y;
+    v[q] = make_float2(c0[q].x + c1[q].x, c0[q].y + c1[q].y);
+    v[4 + q] = make_float2(ar * dx - ai * dy, ar * dy + ai * dx);
+  }
+}
+
 // weights_point for a BCC cell in complex64 from its row constants rc and x frequency k
 // (G^ as in evolve_bcc_row): acc[0] += |c0|^2 + |c1|^2, acc[1] += c0^dag G^_q0 c0 +
 // c1^dag G^_q1 c1 with G^_q1 = -Gamma G^_q0 Gamma.
@@ -768,12 +945,12 @@ __device__ __forceinline__ void weights_bcc_row(const AxesDev& a, int k, float4 
 }
 
 // Fused x pass of the Fourier form (complex64): for RW rows of every component
-// plane, the forward DFT along x, D_k^t per wave vector (BCC coset mix included)
-// and the inverse DFT along x, with one read and one write of those rows.  The y
+// plane, the forward DFT along x, D_k^t per wave vector (BCC coset mix included; with FW the
+// Foldy-Wouthuysen coefficients instead) and the inverse DFT along x, with one read and one write of those rows.  The y
 // and z transforms run as ordinary passes before and after (transforms along
 // different axes commute).  Needs the x axis in one register pass of length
 // L = R1 * R2 (natural order along x); y, z may be digit-permuted (freq_of).
-template <int R1, int R2>
+template <int R1, int R2, bool FW = false>
 __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int64_t count, Mass ms,
                                                       const double* __restrict__ omega, TimeArg ta, float scale_in,
                                                       const double* __restrict__ norm0, float2* __restrict__ data,
@@ -790,7 +967,7 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
   const int CU = RW * P;                    // lines in use
   const int64_t nrows = count / L;          // rows per plane
   const int64_t row0 = (int64_t)blockIdx.x * RW;
-  const bool bcc_rows = dim == 3 && omega != nullptr;
+  const bool bcc_rows = dim == 3 && (FW || omega != nullptr);
   const int tid = threadIdx.x, c = tid % C, r = tid / C;
   const TwRow<V> tw{tw_line, r};
   // ---- load (cp.async): consecutive threads read consecutive x of one line; line cc = w P + p
@@ -824,7 +1001,10 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
       V v[8];
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp) v[pp] = sm[w * 8 + pp + CP * k];
-      evolve_bcc_row(a, k, rowc[w], ms, nu_tab, row * L + k, ta, scale, v);
+      if constexpr (FW)
+        fw_bcc_row(a, k, rowc[w], ms, scale, v);
+      else
+        evolve_bcc_row(a, k, rowc[w], ms, nu_tab, row * L + k, ta, scale, v);
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp) sm[w * 8 + pp + CP * k] = v[pp];
     }
@@ -839,7 +1019,10 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp)
         if (pp < P) v[pp] = sm[w * P + pp + CP * k];
-      evolve_point<float>(dim, a, k, yy, zz, row * L + k, ms, omega, ta, scale, v);
+      if constexpr (FW)
+        fw_point<float>(dim, a, k, yy, zz, ms, scale, v);
+      else
+        evolve_point<float>(dim, a, k, yy, zz, row * L + k, ms, omega, ta, scale, v);
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp)
         if (pp < P) sm[w * P + pp + CP * k] = v[pp];
@@ -860,9 +1043,9 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
   }
 }
 
-template <int R1, int R2>
-qw_status launch_fused(const Geometry& g, const SpecAxes& ax, double n, double m, const double* omega,
-                              int64_t t, void* psi, const void* tw_line, cudaStream_t st, const double* norm0) {
+template <int R1, int R2, bool FW>
+qw_status launch_fused_op(const Geometry& g, const SpecAxes& ax, double n, double m, const double* omega, int64_t t,
+                          void* psi, const void* tw_line, cudaStream_t st, const double* norm0) {
   constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = 256 / TPL;
   constexpr int CP = (C % 2 == 0) ? C + 1 : C;
   const int P = g.dim == 1 ? 2 : (g.dim == 2 ? 4 : 8);
@@ -870,13 +1053,25 @@ qw_status launch_fused(const Geometry& g, const SpecAxes& ax, double n, double m
   const int64_t nrows = g.vol / L;
   const int64_t grid = (nrows + RW - 1) / RW;
   const size_t smem = fused_rowc_offset(L, CP) + 8 * sizeof(float4);  // lines, then up to 8 row constants
-  const qw_status sa = smem_attr(fused_x_kernel<R1, R2>, (int)smem);
+  const qw_status sa = smem_attr(fused_x_kernel<R1, R2, FW>, (int)smem);
   if (sa != QW_OK) return sa;
-  fused_x_kernel<R1, R2><<<(unsigned)grid, 256, smem, st>>>(
+  fused_x_kernel<R1, R2, FW><<<(unsigned)grid, 256, smem, st>>>(
       g.dim, to_dev(ax), g.vol, make_mass(n, m), omega, make_time(t), (float)(1.0 / (double)g.vol), norm0,
       static_cast<float2*>(psi), static_cast<const float2*>(tw_line));
   QW_CHECK_LAUNCH("fused x pass launch");
   return QW_OK;
+}
+
+template <int R1, int R2>
+qw_status launch_fused(const Geometry& g, const SpecAxes& ax, double n, double m, const double* omega, int64_t t,
+                       void* psi, const void* tw_line, cudaStream_t st, const double* norm0) {
+  return launch_fused_op<R1, R2, false>(g, ax, n, m, omega, t, psi, tw_line, st, norm0);
+}
+
+template <int R1, int R2>
+qw_status launch_fused_fw(const Geometry& g, const SpecAxes& ax, double n, double m, void* psi, const void* tw_line,
+                          cudaStream_t st) {
+  return launch_fused_op<R1, R2, true>(g, ax, n, m, nullptr, 0, psi, tw_line, st, nullptr);
 }
 
 // Particle-weight sums of a spectrum whose remaining transform is the x DFT (complex64):
@@ -1005,11 +1200,15 @@ qw_status launch_weights_x(const Geometry& g, const SpecAxes& ax, double n, doub
   template qw_status launch_fused<A, B>(const Geometry&, const SpecAxes&, double, double, const double*,  \
                                         int64_t, void*, const void*, cudaStream_t, const double*);         \
   template qw_status launch_weights_x<A, B>(const Geometry&, const SpecAxes&, double, double, const void*, \
-                                            const void*, double*, cudaStream_t);
+                                            const void*, double*, cudaStream_t);                               \
+  template qw_status launch_fused_fw<A, B>(const Geometry&, const SpecAxes&, double, double, void*,           \
+                                           const void*, cudaStream_t);
 #define QW_FUSED_X_EXTERN(LEN, A, B)                                                                               \
   extern template qw_status launch_fused<A, B>(const Geometry&, const SpecAxes&, double, double, const double*,  \
                                                int64_t, void*, const void*, cudaStream_t, const double*);         \
   extern template qw_status launch_weights_x<A, B>(const Geometry&, const SpecAxes&, double, double, const void*, \
-                                                   const void*, double*, cudaStream_t);
+                                                   const void*, double*, cudaStream_t);                               \
+  extern template qw_status launch_fused_fw<A, B>(const Geometry&, const SpecAxes&, double, double, void*,          \
+                                                  const void*, cudaStream_t);
 
 }  // namespace qw
