@@ -352,6 +352,10 @@ qw_status launch_position_moments(const Geometry& g, qw_dtype dt, const void* ps
   else
     launch_moments_t<double>(g, psi, partials, st);
   QW_CHECK_LAUNCH("moments launch");
+  return launch_fold_moments(partials, result, st);
+}
+
+qw_status launch_fold_moments(const double* partials, double* result, cudaStream_t st) {
   fold_partials_kernel<<<1, kObsThreads, 0, st>>>(partials, kObsBlocks, result);
   QW_CHECK_LAUNCH("fold launch");
   return QW_OK;

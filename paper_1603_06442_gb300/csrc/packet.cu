@@ -4,6 +4,8 @@
 // inputs here so that no field crosses the host link.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "qw_internal.cuh"
 
 namespace qw {
@@ -92,10 +94,169 @@ __global__ void __launch_bounds__(256) packet_kernel(Geometry g, PacketArgs pa, 
   }
 }
 
+// ---- complex64 without FP64: an FP64 instruction costs ~64 FP32 ones here, and a chain has an axis
+// factor per site (25 FP64 instructions for 16 written bytes: N = 2^27 at 0.4 of 6.8 TB/s).
+// Positions are whole numbers: with x0 = X + delta, d = di - delta for the whole number
+// di = minimum image of pos - X.  The phase k0 d / 2 pi is taken in 64-bit fixed point (turns, modulo
+// 1: exact up to the rounding of k0 / 2 pi), d^2 / (4 sigma^2) from di in two FP32 pieces.
+struct AxisF {
+  long long X, N, wrap;     // floor(x0) mod N, the side, the first image (pos - X) mod N that is taken as - N
+  unsigned long long k, k0; // k0 / 2 pi and delta k0 / 2 pi, in units of 2^-64 turns
+  float dh, dl, ch, cl;     // delta = dh + dl; 1 / (4 sigma^2) = ch + cl
+};
+struct PacketF {
+  AxisF ax[3];
+  float2 chi[4];
+};
+
+static unsigned long long turns64(double t) {
+  t -= floor(t);
+  return t >= 1.0 ? 0ull : (unsigned long long)(t * 18446744073709551616.0);
+}
+
+static AxisF axis_f(double x0, double N, double k0, double inv4s2) {
+  AxisF a;
+  double X = floor(x0);
+  const double delta = x0 - X;
+  X -= N * floor(X / N);
+  a.N = (long long)N;
+  a.X = (long long)X % a.N;
+  if (a.X < 0) a.X += a.N;  // the quotient was rounded up
+  a.wrap = (long long)ceil(0.5 * N + delta);
+  const double kt = k0 / 6.283185307179586232;
+  a.k = turns64(kt);
+  a.k0 = turns64(kt * delta);
+  a.dh = (float)delta;
+  a.dl = (float)(delta - (double)a.dh);
+  a.ch = (float)inv4s2;
+  a.cl = (float)(inv4s2 - (double)a.ch);
+  return a;
+}
+
+__device__ __forceinline__ float2 axis_factor_f(const AxisF& a, long long pos) {
+  long long e = pos - a.X;
+  if (e < 0) e += a.N;
+  const long long di = e >= a.wrap ? e - a.N : e;
+  const unsigned long long turns = (unsigned long long)di * a.k - a.k0;
+  const float t = (float)(int)(turns >> 32) * 2.3283064365386963e-10f;  // in [-1/2, 1/2)
+  float sn, cs;
+  sincospif(2.0f * t, &sn, &cs);
+  const float h = (float)di, l = (float)(di - (long long)h) - a.dh;
+  const float d = h + l, r = (l - (d - h)) - a.dl;  // di - delta = d + r, |r| below an ulp of d
+  const float p = d * d, pe = fmaf(2.0f * d, r, fmaf(d, d, -p));
+  const float arg = fmaf(p, a.ch, fmaf(p, a.cl, pe * a.ch));
+  const float ex = arg < 104.0f ? expf(-arg) : 0.0f;
+  return make_float2(ex * cs, ex * sn);
+}
+
+// Rows of 256 sites (chain) or kPacketGroup rows of the box per unit; a CTA takes units in turn and
+// leaves sum |psi|^2 of what it wrote in partials (four doubles, the last three 0).
+constexpr int kPacketGroup = 16, kPacketChain = 8;
+__global__ void __launch_bounds__(256) packet_f_kernel(Geometry g, PacketF pa, int bx, int64_t units,
+                                                       float2* __restrict__ psi, double* __restrict__ partials) {
+  __shared__ float2 fyz[kPacketGroup];
+  double acc[1] = {0.0};
+  const int tid = threadIdx.x;
+  if (g.dim == 1) {
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+      float sum = 0.f;
+#pragma unroll 2
+      for (int j = 0; j < kPacketChain; ++j) {
+        const int64_t x = (u * kPacketChain + j) * 256 + tid;
+        if (x >= g.nx) break;
+        const float2 f = axis_factor_f(pa.ax[0], x);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const float2 v = cx_mul(f, pa.chi[q]);
+          psi[q * g.vol + x] = v;
+          sum = fmaf(v.x, v.x, fmaf(v.y, v.y, sum));
+        }
+      }
+      acc[0] += (double)sum;
+    }
+  } else {
+    const int tx = tid % bx, ty = tid / bx, by = 256 / bx;
+    const int xt = (int)((g.nx + bx - 1) / bx);
+    const int64_t rows = (int64_t)g.ncoset * g.nz * g.ny;
+    const int scale = g.dim == 3 ? 2 : 1;
+    for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+      const int64_t row0 = u / xt * kPacketGroup;
+      const int x = (int)(u % xt) * bx + tx;
+      __syncthreads();  // fyz of the unit before has been read
+      if (tid < kPacketGroup && row0 + tid < rows) {
+        const int64_t row = row0 + tid, zc = row / g.ny, y = row - zc * g.ny;
+        const int c = (int)(zc / g.nz);
+        float2 f = axis_factor_f(pa.ax[1], scale * y + c);
+        if (g.dim == 3) f = cx_mul(f, axis_factor_f(pa.ax[2], scale * (zc - c * g.nz) + c));
+        fyz[tid] = f;
+      }
+      __syncthreads();
+      if (ty < by && x < g.nx) {
+        float sum = 0.f;
+        int cx = -1;
+        float2 fx = make_float2(0.f, 0.f);
+        for (int r = ty; r < kPacketGroup && row0 + r < rows; r += by) {
+          const int64_t row = row0 + r;
+          const int c = g.ncoset == 2 && row >= g.nz * g.ny ? 1 : 0;
+          if (c != cx) {  // the x factor of the row's coset
+            fx = axis_factor_f(pa.ax[0], (long long)scale * x + c);
+            cx = c;
+          }
+          const float2 f = cx_mul(fx, fyz[r]);
+          float2* dst = psi + (int64_t)c * 3 * g.vol + row * g.nx + x;  // row counts through both cosets
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const float2 v = cx_mul(f, pa.chi[q]);
+            dst[q * g.vol] = v;
+            sum = fmaf(v.x, v.x, fmaf(v.y, v.y, sum));
+          }
+        }
+        acc[0] += (double)sum;
+      }
+    }
+  }
+  if (!partials) return;
+  block_sum<1, 256>(acc);
+  if (tid == 0) {
+    partials[4 * blockIdx.x] = acc[0];
+    partials[4 * blockIdx.x + 1] = partials[4 * blockIdx.x + 2] = partials[4 * blockIdx.x + 3] = 0.0;
+  }
+}
+
+static qw_status launch_packet_f(const Geometry& g, const double* x0, double sigma, const double* k0,
+                                 const double* chi, void* psi, double* partials, cudaStream_t st) {
+  PacketF pa;
+  const double inv4s2 = 1.0 / (4.0 * sigma * sigma);
+  for (int j = 0; j < 3; ++j) pa.ax[j] = axis_f(j < g.dim ? x0[j] : 0.0, (double)g.N, j < g.dim ? k0[j] : 0.0, inv4s2);
+  for (int q = 0; q < 4; ++q) pa.chi[q] = make_float2((float)chi[2 * q], (float)chi[2 * q + 1]);
+  const int bx = (int)(g.nx < 256 ? (g.nx + 31) / 32 * 32 : 256);
+  int64_t units;
+  if (g.dim == 1)
+    units = (g.nx + 256 * kPacketChain - 1) / (256 * kPacketChain);
+  else
+    units = ((int64_t)g.ncoset * g.nz * g.ny + kPacketGroup - 1) / kPacketGroup * ((g.nx + bx - 1) / bx);
+  packet_f_kernel<<<kObsBlocks, 256, 0, st>>>(g, pa, bx, units, static_cast<float2*>(psi), partials);
+  QW_CHECK_LAUNCH("packet launch");
+  return QW_OK;
+}
+
+// Finite parameters in the range of the fixed-point form: a whole number floor(x0), d^2 / (4 sigma^2)
+// within FP32.
+bool packet_sums(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0) {
+  bool ok = dt == QW_C64 && sigma > 1e-6;
+  for (int j = 0; j < g.dim; ++j) ok = ok && fabs(x0[j]) < 9.0e15 && fabs(k0[j]) < 1.0e6;
+  return ok;
+}
+
 qw_status launch_packet(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0,
-                        const double* chi, void* psi, cudaStream_t st) {
+                        const double* chi, void* psi, cudaStream_t st, double* partials) {
   if (!(sigma > 0.0)) {
     set_error("packet: sigma must be > 0");
+    return QW_EINVAL;
+  }
+  if (packet_sums(g, dt, x0, sigma, k0)) return launch_packet_f(g, x0, sigma, k0, chi, psi, partials, st);
+  if (partials) {
+    set_error("packet: no norm for these parameters");
     return QW_EINVAL;
   }
   PacketArgs pa;

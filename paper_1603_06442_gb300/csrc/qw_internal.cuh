@@ -272,8 +272,23 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
 // psi(x) = exp(-|d|^2 / (4 sigma^2)) exp(i k0.d) chi with d the minimum-image
 // displacement from x0 on the periodic box (physical BCC coordinates, lattice
 // coordinates in 2D); chi = s complex values (re, im interleaved).  Not normalised.
+// partials (only where packet_sums; may be null): 4 * kObsBlocks doubles, sum |psi|^2 per CTA in
+// the first of each four (folded as position moments are).
 qw_status launch_packet(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0,
-                        const double* chi, void* psi, cudaStream_t st);
+                        const double* chi, void* psi, cudaStream_t st, double* partials = nullptr);
+// D_k^t as launch_evolve_pointwise and the particle-weight sums as launch_particle_weights of the result, in one
+// pass (complex64, omega_k computed in the kernel); partials: 4 * kObsBlocks doubles.
+qw_status launch_evolve_weights(const Geometry& g, const SpecAxes& ax, double n, double m, int64_t t, void* psi_hat,
+                                const double* norm0, double* partials, double* result, cudaStream_t st);
+// The same on a spectrum whose x axis is still to be transformed: x DFT, D_k^t, weights and inverse x DFT in one
+// pass over the field (where fused_x_supported); partials as for launch_weights_fused_x.
+qw_status launch_evolve_weights_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
+                                        int64_t t, void* psi, const double* norm0, double* partials, double* result,
+                                        cudaStream_t st);
+// Whether launch_packet takes the FP32 path, which can sum |psi|^2.
+bool packet_sums(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0);
+// Fold the per-CTA sums of launch_packet into result (4 doubles).
+qw_status launch_fold_moments(const double* partials, double* result, cudaStream_t st);
 // (sum |psi^|^2, sum psi^dag G/sin(omega) psi^) over the zone into result[0..1].
 // ---- probability projections (projection.cu) ---------------------------------
 // keep: bit 0 x, bit 1 y, bit 2 z.  projection_partials: doubles of chunk partials the

@@ -233,6 +233,66 @@ __global__ void __launch_bounds__(256) weights_kernel(int dim, AxesDev a, int64_
   }
 }
 
+// D_k^t and the particle-weight sums of the evolved values in one pass over the field (served
+// requests): the weights' own pass read the field again and formed every symbol again (BCC, 41
+// requests: 7.6 + 6.0 ms as two passes).
+template <int DIM>
+__global__ void __launch_bounds__(256, DIM == 3 ? 2 : 3)
+    evolve_weights_kernel(AxesDev a, int64_t count, Mass ms, TimeArg ta, float scale_in,
+                          const double* __restrict__ norm0, float2* __restrict__ data, double* __restrict__ partials) {
+  constexpr int P = DIM == 1 ? 2 : DIM == 2 ? 4 : 8;
+  constexpr int U = 8 / P;  // points per round: 64 bytes of loads in flight per thread on every lattice
+  const float scale = norm0 ? scale_in * rsqrtf((float)norm0[0]) : scale_in;
+  const int64_t nx = a.len[0], ny = a.len[1], stride = (int64_t)gridDim.x * 256;
+  double acc[2] = {0.0, 0.0};
+  float seg[2] = {0.f, 0.f};  // segments of 16 points summed in FP32, segment sums in FP64
+  int nseg = 0;
+  for (int64_t base = (int64_t)blockIdx.x * 256 + threadIdx.x; base < count; base += U * stride) {
+    float2 v[U][8];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t idx = base + u * stride;
+#pragma unroll
+      for (int q = 0; q < P; ++q)
+        if (idx < count) v[u][q] = data[q * count + idx];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int64_t idx = base + u * stride;
+      if (idx >= count) break;
+      int64_t x = idx, y = 0, z = 0;
+      if (DIM > 1 && count <= 0x7fffffff) {  // 32-bit index arithmetic for planes below 2^31 values
+        const int i32 = (int)idx, nx32 = (int)nx, ny32 = (int)ny;
+        const int yz = i32 / nx32;
+        x = i32 - yz * nx32;
+        y = yz % ny32;
+        z = yz / ny32;
+      } else if (DIM > 1) {
+        x = idx % nx;
+        y = (idx / nx) % ny;
+        z = idx / (nx * ny);
+      }
+      evolve_point<float>(DIM, a, x, y, z, idx, ms, nullptr, ta, scale, v[u]);
+#pragma unroll
+      for (int q = 0; q < P; ++q) data[q * count + idx] = v[u][q];
+      weights_point<float>(DIM, a, x, y, z, ms, v[u], seg);
+      if (++nseg == 16) {
+        acc[0] += (double)seg[0];
+        acc[1] += (double)seg[1];
+        seg[0] = seg[1] = 0.f;
+        nseg = 0;
+      }
+    }
+  }
+  acc[0] += (double)seg[0];
+  acc[1] += (double)seg[1];
+  block_sum<2, 256>(acc);
+  if (threadIdx.x == 0) {
+    partials[2 * blockIdx.x] = acc[0];
+    partials[2 * blockIdx.x + 1] = acc[1];
+  }
+}
+
 // Sum of nblk (a, b) partial pairs in a fixed order: 1024 threads, four independent
 // accumulators per thread (the partial count reaches 10^5 for the x-pass weights).
 constexpr int kFoldThreads = 1024;
@@ -335,6 +395,27 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
                            count, make_mass(n, m), omega, make_time(t), inv, norm0, static_cast<double2*>(psi_hat));
 }
 
+template <int DIM>
+static qw_status evolve_weights_dim(const AxesDev& a, int64_t count, double n, double m, int64_t t, float scale,
+                                    float2* psi_hat, const double* norm0, double* partials, double* result,
+                                    cudaStream_t st) {
+  const int resident = resident_blocks(evolve_weights_kernel<DIM>, 256);
+  const int nblk = resident > 0 && resident < 2 * kObsBlocks ? resident : 2 * kObsBlocks;
+  evolve_weights_kernel<DIM><<<nblk, 256, 0, st>>>(a, count, make_mass(n, m), make_time(t), scale, norm0, psi_hat,
+                                                   partials);
+  QW_CHECK_LAUNCH("evolve and weights launch");
+  fold2_kernel<<<1, kFoldThreads, 0, st>>>(partials, nblk, result);
+  QW_CHECK_LAUNCH("fold launch");
+  return QW_OK;
+}
+
+qw_status launch_evolve_weights(const Geometry& g, const SpecAxes& ax, double n, double m, int64_t t, void* psi_hat,
+                                const double* norm0, double* partials, double* result, cudaStream_t st) {
+  auto* run = g.dim == 1 ? evolve_weights_dim<1> : g.dim == 2 ? evolve_weights_dim<2> : evolve_weights_dim<3>;
+  return run(to_dev(ax), kcount(g), n, m, t, (float)(1.0 / (double)g.vol), static_cast<float2*>(psi_hat), norm0,
+             partials, result, st);
+}
+
 qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m, void* psi_hat,
                               cudaStream_t st) {
   const int64_t count = kcount(g);
@@ -420,6 +501,27 @@ qw_status launch_weights_fused_x(const Geometry& g, const SpecAxes& ax, const Ff
   }
   if (s2 != QW_OK) return s2;
   // partials holds 2 * (CTAs + kFoldCtas) doubles: the CTAs' pairs, then the fold's first stage
+  const int64_t nblk = fused_x_grid(g);
+  return launch_fold_partials(partials, nblk, 2, partials + 2 * nblk, result, st);
+}
+
+qw_status launch_evolve_weights_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
+                                        int64_t t, void* psi, const double* norm0, double* partials, double* result,
+                                        cudaStream_t st) {
+  const void* tw = f.pass[f.axis[0].first].tw_line;
+  qw_status s2 = QW_OK;
+  switch (g.nx) {
+#define QW_FX(LEN, A, B)                                                                           \
+  case LEN:                                                                                        \
+    s2 = launch_fused_evolve_weights<A, B>(g, ax, n, m, t, psi, tw, st, norm0, partials); \
+    break;
+    QW_FUSED_LENGTHS(QW_FX)
+#undef QW_FX
+    default:
+      set_error("fused x pass: no register kernel for length %lld", (long long)g.nx);
+      return QW_EINVAL;
+  }
+  if (s2 != QW_OK) return s2;
   const int64_t nblk = fused_x_grid(g);
   return launch_fold_partials(partials, nblk, 2, partials + 2 * nblk, result, st);
 }
