@@ -243,14 +243,12 @@ SpecAxes spec_axes(const Geometry& g, const FftPlan& f);
 qw_status launch_omega_table(const Geometry& g, const SpecAxes& ax, double n, double m, double* omega,
                              cudaStream_t st, bool split);
 // psi_hat (forward DFT, storage order) <- D_k^t psi_hat / |V|, BCC cosets mixed per cell;
-// with norm0 (device, optional) the result is also divided by sqrt(norm0[0]);
 // omega == nullptr computes omega_k in the kernel (FP64) instead of reading a table.
 // Fused x pass: forward DFT along x, D_k^t, inverse DFT along x (complex64, 2D/BCC,
 // x axis in one register pass); y and z are transformed around it by the caller.
 bool fused_x_supported(const Geometry& g, const FftPlan& f, qw_dtype dt);
 qw_status launch_evolve_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
-                                const double* omega, int64_t t, void* psi, cudaStream_t st,
-                                const double* norm0 = nullptr);
+                                const double* omega, int64_t t, void* psi, cudaStream_t st);
 // With the same tiling, the particle-weight sums of a spectrum still to be transformed
 // along x (complex64): 2 doubles per CTA (fused_x_grid CTAs) into partials, folded into
 // result[0..1] through the 2 * kFoldCtas doubles after them; data is only read.
@@ -265,8 +263,7 @@ qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt
 qw_status launch_fw_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m, void* psi,
                             cudaStream_t st);
 qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m,
-                                  const double* omega, int64_t t, void* psi_hat, cudaStream_t st,
-                                  const double* norm0 = nullptr);
+                                  const double* omega, int64_t t, void* psi_hat, cudaStream_t st);
 
 // ---- state preparation (packet.cu) ---------------------------------------------
 // psi(x) = exp(-|d|^2 / (4 sigma^2)) exp(i k0.d) chi with d the minimum-image
@@ -277,14 +274,10 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
 qw_status launch_packet(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0,
                         const double* chi, void* psi, cudaStream_t st, double* partials = nullptr);
 // D_k^t as launch_evolve_pointwise and the particle-weight sums as launch_particle_weights of the result, in one
-// pass (complex64, omega_k computed in the kernel); partials: 4 * kObsBlocks doubles.
+// pass (complex64, omega_k computed in the kernel; the result is also divided by sqrt(norm0[0]));
+// partials: 4 * kObsBlocks doubles.
 qw_status launch_evolve_weights(const Geometry& g, const SpecAxes& ax, double n, double m, int64_t t, void* psi_hat,
                                 const double* norm0, double* partials, double* result, cudaStream_t st);
-// The same on a spectrum whose x axis is still to be transformed: x DFT, D_k^t, weights and inverse x DFT in one
-// pass over the field (where fused_x_supported); partials as for launch_weights_fused_x.
-qw_status launch_evolve_weights_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
-                                        int64_t t, void* psi, const double* norm0, double* partials, double* result,
-                                        cudaStream_t st);
 // Whether launch_packet takes the FP32 path, which can sum |psi|^2.
 bool packet_sums(const Geometry& g, qw_dtype dt, const double* x0, double sigma, const double* k0);
 // Fold the per-CTA sums of launch_packet into result (4 doubles).

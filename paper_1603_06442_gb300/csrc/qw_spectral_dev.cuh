@@ -944,60 +944,29 @@ __device__ __forceinline__ void weights_bcc_row(const AxesDev& a, int k, float4 
   acc[1] += g;
 }
 
-// The pair of sums of a CTA of 256 threads into partials[2 b], [2 b + 1].  Warp sums in FP32 (64
-// points), the eight warp sums in FP64 in a fixed order: an FP64 block reduction per thread would cost
-// more than the thread's points.
-__device__ __forceinline__ void fold_points(float (&facc)[2], double* __restrict__ partials) {
-  const int tid = threadIdx.x;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    facc[0] += __shfl_xor_sync(0xffffffffu, facc[0], o);
-    facc[1] += __shfl_xor_sync(0xffffffffu, facc[1], o);
-  }
-  __shared__ float wsum[8][2];
-  if ((tid & 31) == 0) {
-    wsum[tid >> 5][0] = facc[0];
-    wsum[tid >> 5][1] = facc[1];
-  }
-  __syncthreads();
-  if (tid == 0) {
-    double a0 = 0.0, a1 = 0.0;
-    for (int w = 0; w < 8; ++w) {
-      a0 += (double)wsum[w][0];
-      a1 += (double)wsum[w][1];
-    }
-    partials[2 * blockIdx.x] = a0;
-    partials[2 * blockIdx.x + 1] = a1;
-  }
-}
-
 // Fused x pass of the Fourier form (complex64): for RW rows of every component
 // plane, the forward DFT along x, D_k^t per wave vector (BCC coset mix included; with FW the
 // Foldy-Wouthuysen coefficients instead) and the inverse DFT along x, with one read and one write of those rows.  The y
 // and z transforms run as ordinary passes before and after (transforms along
 // different axes commute).  Needs the x axis in one register pass of length
 // L = R1 * R2 (natural order along x); y, z may be digit-permuted (freq_of).
-// FUSED_EVOLVE_WEIGHTS (served requests, omega_k computed here) also sums the particle weights of the
-// evolved values: partials[2 b], [2 b + 1] per CTA b.
-enum { FUSED_EVOLVE, FUSED_FW, FUSED_EVOLVE_WEIGHTS };
-template <int R1, int R2, int OP>
-__global__ void __launch_bounds__(256, OP == FUSED_EVOLVE_WEIGHTS ? 2 : 3)
-    fused_x_kernel(int dim, AxesDev a, int64_t count, Mass ms, const double* __restrict__ omega, TimeArg ta,
-                   float scale_in, const double* __restrict__ norm0, float2* __restrict__ data,
-                   const float2* __restrict__ tw_line, double* __restrict__ partials) {
+template <int R1, int R2, bool FW = false>
+__global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int64_t count, Mass ms,
+                                                      const double* __restrict__ omega, TimeArg ta, float scale,
+                                                      float2* __restrict__ data,
+                                                      const float2* __restrict__ tw_line) {
   using V = float2;
   constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = 256 / TPL;
   constexpr int CP = (C % 2 == 0) ? C + 1 : C;
   extern __shared__ __align__(16) unsigned char fx_smem[];
   V* sm = reinterpret_cast<V*>(fx_smem);
   float4* rowc = reinterpret_cast<float4*>(fx_smem + fused_rowc_offset(L, CP));  // BCC row constants
-  const float scale = norm0 ? scale_in * rsqrtf((float)norm0[0]) : scale_in;
   const int P = planes_of(dim);
   const int RW = C / P;                     // rows per CTA (C >= 8 >= P)
   const int CU = RW * P;                    // lines in use
   const int64_t nrows = count / L;          // rows per plane
   const int64_t row0 = (int64_t)blockIdx.x * RW;
-  const bool bcc_rows = dim == 3 && (OP == FUSED_FW || (OP == FUSED_EVOLVE && omega != nullptr));
+  const bool bcc_rows = dim == 3 && (FW || omega != nullptr);
   const int tid = threadIdx.x, c = tid % C, r = tid / C;
   const TwRow<V> tw{tw_line, r};
   // ---- load (cp.async): consecutive threads read consecutive x of one line; line cc = w P + p
@@ -1022,7 +991,6 @@ __global__ void __launch_bounds__(256, OP == FUSED_EVOLVE_WEIGHTS ? 2 : 3)
   __syncthreads();
   reg_fft_steps<float, false, R1, R2, CP>(sm, c, r, tw);
   // ---- D_k^t at every (row, k) of the CTA
-  float facc[2] = {0.f, 0.f};  // a thread sums RW L / 256 points (2-4) in FP32
   if (bcc_rows) {
     const float2* nu_tab = reinterpret_cast<const float2*>(omega);
     for (int q = tid; q < RW * L; q += 256) {
@@ -1032,7 +1000,7 @@ __global__ void __launch_bounds__(256, OP == FUSED_EVOLVE_WEIGHTS ? 2 : 3)
       V v[8];
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp) v[pp] = sm[w * 8 + pp + CP * k];
-      if constexpr (OP == FUSED_FW)
+      if constexpr (FW)
         fw_bcc_row(a, k, rowc[w], ms, scale, v);
       else
         evolve_bcc_row(a, k, rowc[w], ms, nu_tab, row * L + k, ta, scale, v);
@@ -1050,11 +1018,10 @@ __global__ void __launch_bounds__(256, OP == FUSED_EVOLVE_WEIGHTS ? 2 : 3)
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp)
         if (pp < P) v[pp] = sm[w * P + pp + CP * k];
-      if constexpr (OP == FUSED_FW)
+      if constexpr (FW)
         fw_point<float>(dim, a, k, yy, zz, ms, scale, v);
       else
         evolve_point<float>(dim, a, k, yy, zz, row * L + k, ms, omega, ta, scale, v);
-      if constexpr (OP == FUSED_EVOLVE_WEIGHTS) weights_point<float>(dim, a, k, yy, zz, ms, v, facc);
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp)
         if (pp < P) sm[w * P + pp + CP * k] = v[pp];
@@ -1073,13 +1040,11 @@ __global__ void __launch_bounds__(256, OP == FUSED_EVOLVE_WEIGHTS ? 2 : 3)
     const int p = cc & (P - 1), w = cc >> lgP;
     if (cc < CU && row0 + w < nrows) data[p * count + (row0 + w) * L + xx] = sm[cc + CP * xx];
   }
-  if constexpr (OP == FUSED_EVOLVE_WEIGHTS) fold_points(facc, partials);
 }
 
-template <int R1, int R2, int OP>
+template <int R1, int R2, bool FW>
 qw_status launch_fused_op(const Geometry& g, const SpecAxes& ax, double n, double m, const double* omega, int64_t t,
-                          void* psi, const void* tw_line, cudaStream_t st, const double* norm0,
-                          double* partials = nullptr) {
+                          void* psi, const void* tw_line, cudaStream_t st) {
   constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = 256 / TPL;
   constexpr int CP = (C % 2 == 0) ? C + 1 : C;
   const int P = g.dim == 1 ? 2 : (g.dim == 2 ? 4 : 8);
@@ -1087,32 +1052,25 @@ qw_status launch_fused_op(const Geometry& g, const SpecAxes& ax, double n, doubl
   const int64_t nrows = g.vol / L;
   const int64_t grid = (nrows + RW - 1) / RW;
   const size_t smem = fused_rowc_offset(L, CP) + 8 * sizeof(float4);  // lines, then up to 8 row constants
-  const qw_status sa = smem_attr(fused_x_kernel<R1, R2, OP>, (int)smem);
+  const qw_status sa = smem_attr(fused_x_kernel<R1, R2, FW>, (int)smem);
   if (sa != QW_OK) return sa;
-  fused_x_kernel<R1, R2, OP><<<(unsigned)grid, 256, smem, st>>>(
-      g.dim, to_dev(ax), g.vol, make_mass(n, m), omega, make_time(t), (float)(1.0 / (double)g.vol), norm0,
-      static_cast<float2*>(psi), static_cast<const float2*>(tw_line), partials);
+  fused_x_kernel<R1, R2, FW><<<(unsigned)grid, 256, smem, st>>>(
+      g.dim, to_dev(ax), g.vol, make_mass(n, m), omega, make_time(t), (float)(1.0 / (double)g.vol),
+      static_cast<float2*>(psi), static_cast<const float2*>(tw_line));
   QW_CHECK_LAUNCH("fused x pass launch");
   return QW_OK;
 }
 
 template <int R1, int R2>
 qw_status launch_fused(const Geometry& g, const SpecAxes& ax, double n, double m, const double* omega, int64_t t,
-                       void* psi, const void* tw_line, cudaStream_t st, const double* norm0) {
-  return launch_fused_op<R1, R2, FUSED_EVOLVE>(g, ax, n, m, omega, t, psi, tw_line, st, norm0);
+                       void* psi, const void* tw_line, cudaStream_t st) {
+  return launch_fused_op<R1, R2, false>(g, ax, n, m, omega, t, psi, tw_line, st);
 }
 
 template <int R1, int R2>
 qw_status launch_fused_fw(const Geometry& g, const SpecAxes& ax, double n, double m, void* psi, const void* tw_line,
                           cudaStream_t st) {
-  return launch_fused_op<R1, R2, FUSED_FW>(g, ax, n, m, nullptr, 0, psi, tw_line, st, nullptr);
-}
-
-// partials: a pair of doubles per CTA
-template <int R1, int R2>
-qw_status launch_fused_evolve_weights(const Geometry& g, const SpecAxes& ax, double n, double m, int64_t t, void* psi,
-                                      const void* tw_line, cudaStream_t st, const double* norm0, double* partials) {
-  return launch_fused_op<R1, R2, FUSED_EVOLVE_WEIGHTS>(g, ax, n, m, nullptr, t, psi, tw_line, st, norm0, partials);
+  return launch_fused_op<R1, R2, true>(g, ax, n, m, nullptr, 0, psi, tw_line, st);
 }
 
 // Particle-weight sums of a spectrum whose remaining transform is the x DFT (complex64):
@@ -1178,7 +1136,28 @@ __global__ void __launch_bounds__(256, 3) weights_x_kernel(int dim, AxesDev a, i
       weights_point<float>(dim, a, k, yy, zz, ms, v, facc);
     }
   }
-  fold_points(facc, partials);
+  // warp sums in FP32 (64 points), the eight warp sums in FP64 in a fixed order: an FP64
+  // block reduction per thread would cost more than the thread's points here
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    facc[0] += __shfl_xor_sync(0xffffffffu, facc[0], o);
+    facc[1] += __shfl_xor_sync(0xffffffffu, facc[1], o);
+  }
+  __shared__ float wsum[8][2];
+  if ((tid & 31) == 0) {
+    wsum[tid >> 5][0] = facc[0];
+    wsum[tid >> 5][1] = facc[1];
+  }
+  __syncthreads();
+  if (tid == 0) {
+    double a0 = 0.0, a1 = 0.0;
+    for (int w = 0; w < 8; ++w) {
+      a0 += (double)wsum[w][0];
+      a1 += (double)wsum[w][1];
+    }
+    partials[2 * blockIdx.x] = a0;
+    partials[2 * blockIdx.x + 1] = a1;
+  }
 }
 
 // CTAs of the fused x pass and of weights_x_kernel (rows of RW per CTA)
@@ -1217,21 +1196,15 @@ qw_status launch_weights_x(const Geometry& g, const SpecAxes& ax, double n, doub
   QW_FUSED_LENGTHS_1(X) QW_FUSED_LENGTHS_2(X) QW_FUSED_LENGTHS_3(X) QW_FUSED_LENGTHS_4(X) \
   QW_FUSED_LENGTHS_5(X) QW_FUSED_LENGTHS_6(X)
 #define QW_FUSED_X_INSTANTIATE(LEN, A, B)                                                                     \
-  template qw_status launch_fused_evolve_weights<A, B>(const Geometry&, const SpecAxes&, double, double,      \
-                                                       int64_t, void*, const void*, cudaStream_t,            \
-                                                       const double*, double*);                              \
   template qw_status launch_fused<A, B>(const Geometry&, const SpecAxes&, double, double, const double*,  \
-                                        int64_t, void*, const void*, cudaStream_t, const double*);         \
+                                        int64_t, void*, const void*, cudaStream_t);                        \
   template qw_status launch_weights_x<A, B>(const Geometry&, const SpecAxes&, double, double, const void*, \
                                             const void*, double*, cudaStream_t);                               \
   template qw_status launch_fused_fw<A, B>(const Geometry&, const SpecAxes&, double, double, void*,           \
                                            const void*, cudaStream_t);
 #define QW_FUSED_X_EXTERN(LEN, A, B)                                                                               \
-  extern template qw_status launch_fused_evolve_weights<A, B>(const Geometry&, const SpecAxes&, double, double,    \
-                                                              int64_t, void*, const void*, cudaStream_t,          \
-                                                              const double*, double*);                            \
   extern template qw_status launch_fused<A, B>(const Geometry&, const SpecAxes&, double, double, const double*,  \
-                                               int64_t, void*, const void*, cudaStream_t, const double*);         \
+                                               int64_t, void*, const void*, cudaStream_t);                        \
   extern template qw_status launch_weights_x<A, B>(const Geometry&, const SpecAxes&, double, double, const void*, \
                                                    const void*, double*, cudaStream_t);                               \
   extern template qw_status launch_fused_fw<A, B>(const Geometry&, const SpecAxes&, double, double, void*,          \

@@ -20,7 +20,6 @@
 // state and, once done, the observables and the submit-to-done latency.
 #include <cuda_runtime.h>
 
-#include <algorithm>
 #include <chrono>
 #include <cmath>
 #include <condition_variable>
@@ -138,7 +137,6 @@ struct qw_server_s {
   int device = 0;
   size_t budget = 0;
   void* pool_base = nullptr;
-  int64_t part_doubles = 0;  // doubles in each slot's d_part
   Pool pool;
   std::vector<Slot> slots;
   size_t max_pending = 0;
@@ -251,22 +249,13 @@ static qw_status launch_request(qw_server_s* S, Slot& sl) {
   st = summed ? launch_fold_moments(sl.d_part, sl.d_res, s)
               : launch_position_moments(g, QW_C64, psi, sl.d_part, sl.d_res, s);
   if (st != QW_OK) return st;
+  if ((st = fft_forward(*f, g.dim, psi, s)) != QW_OK) return st;
   // D_k^t with omega_k computed in the kernel (a request's table would be used once), and the
   // particle weights of the evolved spectrum: |P(+-) psi^_k|^2 is what a forward DFT of psi(t)
   // would give (the ratio does not depend on the DFT's scale)
-  if (fused_x_supported(g, *f, QW_C64) && 2 * (fused_x_grid(g) + kFoldCtas) <= S->part_doubles) {  // between the two x transforms, in their pass
-    for (int j = g.dim - 1; j >= 1; --j)
-      if ((st = fft_forward_axis(*f, j, psi, s)) != QW_OK) return st;
-    st = launch_evolve_weights_fused_x(g, ax, *f, n, m, R.req.t, psi, sl.d_res, sl.d_part, sl.d_res + 8, s);
-    if (st != QW_OK) return st;
-    for (int j = 1; j < g.dim; ++j)
-      if ((st = fft_inverse_axis(*f, j, psi, s)) != QW_OK) return st;
-  } else {
-    if ((st = fft_forward(*f, g.dim, psi, s)) != QW_OK) return st;
-    st = launch_evolve_weights(g, ax, n, m, R.req.t, psi, sl.d_res, sl.d_part, sl.d_res + 8, s);
-    if (st != QW_OK) return st;
-    if ((st = fft_inverse(*f, g.dim, psi, s)) != QW_OK) return st;
-  }
+  st = launch_evolve_weights(g, ax, n, m, R.req.t, psi, sl.d_res, sl.d_part, sl.d_res + 8, s);
+  if (st != QW_OK) return st;
+  if ((st = fft_inverse(*f, g.dim, psi, s)) != QW_OK) return st;
   if ((st = launch_position_moments(g, QW_C64, psi, sl.d_part, sl.d_res + 4, s)) != QW_OK) return st;
   QW_CHECK_CUDA(cudaMemcpyAsync(sl.h_res, sl.d_res, 10 * sizeof(double), cudaMemcpyDeviceToHost, s));
   QW_CHECK_CUDA(cudaEventRecord(sl.done, s));
@@ -372,15 +361,13 @@ qw_status qw_server_create(size_t hbm_budget_bytes, int slots, int max_pending, 
   S->max_pending = (size_t)max_pending;
   cudaError_t e = cudaGetDevice(&S->device);
   if (e == cudaSuccess) e = cudaMalloc(&S->pool_base, hbm_budget_bytes);
-  // a fused x pass leaves a pair of sums per CTA, at most one per 10 KB of the field and 2^18 of them
-  S->part_doubles = std::max<int64_t>(4 * kObsBlocks, 2 * (std::min<int64_t>(1 << 18, hbm_budget_bytes / 10000) + kFoldCtas));
   S->pool.init(hbm_budget_bytes);
   S->slots.resize(slots);
   for (auto& sl : S->slots) {
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&sl.stream, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(&sl.done, cudaEventDisableTiming);
     if (e == cudaSuccess) e = cudaMalloc(&sl.d_res, 16 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&sl.d_part, S->part_doubles * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&sl.d_part, 4 * kObsBlocks * sizeof(double));
     if (e == cudaSuccess) e = cudaMallocHost(&sl.h_res, 16 * sizeof(double));
   }
   if (e != cudaSuccess) {

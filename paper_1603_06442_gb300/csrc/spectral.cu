@@ -141,15 +141,10 @@ __global__ void omega_dd_kernel(int dim, AxesDev a, double m, const double2* __r
 
 template <typename T>
 __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t count, Mass ms,
-                                                     const double* __restrict__ omega, TimeArg ta, T scale_in,
-                                                     const double* __restrict__ norm0,
+                                                     const double* __restrict__ omega, TimeArg ta, T scale,
                                                      typename Cx2<T>::t* __restrict__ data) {
   using V = typename Cx2<T>::t;
   grid_wait();
-  // optional normalisation of the initial state, folded into the 1/|V| scale
-  const T scale = norm0 ? (sizeof(T) == 8 ? (T)((double)scale_in / sqrt(norm0[0]))
-                                           : (T)(scale_in * rsqrtf((float)norm0[0])))
-                        : scale_in;
   int64_t x, y, z;
   if (grid_pos(a, x, y, z)) {
     const int64_t idx = (z * a.len[1] + y) * a.len[0] + x;
@@ -234,8 +229,10 @@ __global__ void __launch_bounds__(256) weights_kernel(int dim, AxesDev a, int64_
 }
 
 // D_k^t and the particle-weight sums of the evolved values in one pass over the field (served
-// requests): the weights' own pass read the field again and formed every symbol again (BCC, 41
-// requests: 7.6 + 6.0 ms as two passes).
+// requests): the weights' own pass read the field again and formed every symbol again (7.6 + 6.0 ms
+// of a burst of 48 requests as two passes).  Bound by the arithmetic of omega_k and the symbol more than
+// by HBM, so it is not put inside the fused x pass: with the x transforms around it there a CTA's loads
+// wait for that arithmetic (the burst: 68.9 ms instead of 65.8, though two passes over the field fewer).
 template <int DIM>
 __global__ void __launch_bounds__(256, DIM == 3 ? 2 : 3)
     evolve_weights_kernel(AxesDev a, int64_t count, Mass ms, TimeArg ta, float scale_in,
@@ -381,18 +378,17 @@ qw_status launch_omega_table(const Geometry& g, const SpecAxes& ax, double n, do
 }
 
 qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt, double n, double m,
-                                  const double* omega, int64_t t, void* psi_hat, cudaStream_t st,
-                                  const double* norm0) {
+                                  const double* omega, int64_t t, void* psi_hat, cudaStream_t st) {
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
   const int threads = point_threads(g, dt);
   const bool overlap = small_field(g, dt);
   if (dt == QW_C64)
     return launch_overlapped(evolve_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
-                             count, make_mass(n, m), omega, make_time(t), (float)inv, norm0,
+                             count, make_mass(n, m), omega, make_time(t), (float)inv,
                              static_cast<float2*>(psi_hat));
   return launch_overlapped(evolve_kernel<double>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
-                           count, make_mass(n, m), omega, make_time(t), inv, norm0, static_cast<double2*>(psi_hat));
+                           count, make_mass(n, m), omega, make_time(t), inv, static_cast<double2*>(psi_hat));
 }
 
 template <int DIM>
@@ -443,12 +439,12 @@ bool fused_x_supported(const Geometry& g, const FftPlan& f, qw_dtype dt) {
 }
 
 qw_status launch_evolve_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
-                                const double* omega, int64_t t, void* psi, cudaStream_t st, const double* norm0) {
+                                const double* omega, int64_t t, void* psi, cudaStream_t st) {
   const void* tw = f.pass[f.axis[0].first].tw_line;
   switch (g.nx) {
 #define QW_FX(LEN, A, B) \
   case LEN:              \
-    return launch_fused<A, B>(g, ax, n, m, omega, t, psi, tw, st, norm0);
+    return launch_fused<A, B>(g, ax, n, m, omega, t, psi, tw, st);
     QW_FUSED_LENGTHS(QW_FX)
 #undef QW_FX
     default:
@@ -501,27 +497,6 @@ qw_status launch_weights_fused_x(const Geometry& g, const SpecAxes& ax, const Ff
   }
   if (s2 != QW_OK) return s2;
   // partials holds 2 * (CTAs + kFoldCtas) doubles: the CTAs' pairs, then the fold's first stage
-  const int64_t nblk = fused_x_grid(g);
-  return launch_fold_partials(partials, nblk, 2, partials + 2 * nblk, result, st);
-}
-
-qw_status launch_evolve_weights_fused_x(const Geometry& g, const SpecAxes& ax, const FftPlan& f, double n, double m,
-                                        int64_t t, void* psi, const double* norm0, double* partials, double* result,
-                                        cudaStream_t st) {
-  const void* tw = f.pass[f.axis[0].first].tw_line;
-  qw_status s2 = QW_OK;
-  switch (g.nx) {
-#define QW_FX(LEN, A, B)                                                                           \
-  case LEN:                                                                                        \
-    s2 = launch_fused_evolve_weights<A, B>(g, ax, n, m, t, psi, tw, st, norm0, partials); \
-    break;
-    QW_FUSED_LENGTHS(QW_FX)
-#undef QW_FX
-    default:
-      set_error("fused x pass: no register kernel for length %lld", (long long)g.nx);
-      return QW_EINVAL;
-  }
-  if (s2 != QW_OK) return s2;
   const int64_t nblk = fused_x_grid(g);
   return launch_fold_partials(partials, nblk, 2, partials + 2 * nblk, result, st);
 }

@@ -58,8 +58,7 @@ def test_packet_outside_the_fixed_point_range(qb, k0, sigma):
     assert np.linalg.norm(got - want) < 1e-6
 
 
-# The weights summed while evolving (several rounds of the resident CTAs with a remainder; x axes with and
-# without the fused x pass) against the plan's own packet, evolution and observables; the tolerances are those
+# The weights summed while evolving (several rounds of the resident CTAs with a remainder) against the plan's own packet, evolution and observables; the tolerances are those
 # of a served request against the oracle.
 @pytest.mark.parametrize("dim,N", [(1, 3 ** 14), (2, 2187), (2, 288), (3, 2 * 81), (3, 2 * 54), (3, 2 * 216)])
 @pytest.mark.parametrize("t", [0, 1, 4321])
