@@ -1,14 +1,14 @@
 // BCC boxes: several steps of the update rule per pass over HBM with the marching kernel of
 // qw_march.cuh (any M, complex64 and complex128), and the choice of its tile per box.
 //
-// complex64, one GB300, G site-steps/s of the kernel against the kernels it replaced (the two-step
-// TMA kernel for M % 64 = 0, one thread per site and step otherwise): M = 256: 214 against 121;
-// M = 125: 168 against 68; M = 64: 79 against 36.  It is bound by issue slots and dependent
+// complex64, one GB300, G site-steps/s against the kernels it replaced (the two-step
+// TMA kernel for M % 64 = 0, one thread per site and step otherwise): M = 256: 206 against 121;
+// M = 125: 166 against 68; M = 64: 90 against 36.  It is bound by issue slots and dependent
 // latencies (2 warps per scheduler at ~250 registers; IPC 0.55, FP32 pipe 40%), no longer by
 // shared memory (40% of the wavefront peak) or HBM (31%), so what a tile recomputes in its halo
 // costs directly: the tile and the number of steps are chosen by the estimate below.
 // complex128: bound by the FP64 pipe (2 lanes a clock and SM): 48 FP64 instructions a site-step
-// instead of 104, one step a launch (every recomputed site costs): M = 64: 7.5 against 5.1.
+// instead of 104, one step a launch (every recomputed site costs): M = 64: 7.9 against 5.1.
 #include <cuda_runtime.h>
 
 #include "qw_march.cuh"
@@ -55,13 +55,23 @@ template <typename C> March3<C> geometry3(const Geometry& g, const Tile3& s, int
   return p;
 }
 
-double estimate3(const Geometry& g, const Tile3& s, int sms) {
+double estimate3(const Geometry& g, const Tile3& s, int elem, int sms) {
   int grid;
   const March3<float2> p = geometry3<float2>(g, s, sms, &grid);
   const int P = 2 * p.g.M;
   int iters = p.rounds * (P + 2 * s.t);
   if (p.rest) iters += (p.planes < P ? p.planes : P) + 2 * s.t;
-  return 2.5 + iters * s.us;  // us a launch: start and end, and the half-layers of the longest CTA
+  const double us = 2.5 + iters * s.us;  // a launch: start and end, and the half-layers of the longest CTA
+  const double field = (double)g.elems * elem;
+  if (field < 64e6) return us;
+  // Fields beyond L2: the boxes read with their halos and the field written, at 5.2 TB/s.  Tiles find
+  // their neighbours' rows in L2 only while the CTAs keep to one height, which the larger boxes do not:
+  // three steps a launch took 545-645 us at N = 512 and 5062 at N = 1024 (450 and 3480 without this
+  // bound), four 638 and 4651, so N = 512 went from 156 to 206 G site-steps/s; at N = 450 three stay
+  // the better choice (322 against 498 us).
+  const double box = (double)p.ntx * p.nty * 32 * s.kx * s.ky * s.nw / ((double)p.g.M * p.g.M);
+  const double hbm = field * (box + 1.0) / 5.2e6;
+  return us > hbm ? us : hbm;
 }
 
 }  // namespace
@@ -72,7 +82,7 @@ double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
   const int n = dt == QW_C64 ? (int)(sizeof(kTiles64) / sizeof(Tile3)) : (int)(sizeof(kTiles128) / sizeof(Tile3));
   for (int i = 0; i < n; ++i)
     if (t[i].t == steps) {
-      const double c = estimate3(g, t[i], sms);
+      const double c = estimate3(g, t[i], dt == QW_C64 ? 8 : 16, sms);
       if (best < 0 || c < best) best = c;
     }
   return best;
@@ -86,7 +96,7 @@ qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, dou
   double bc = 0.0;
   for (int i = 0; i < cnt; ++i) {
     if (t[i].t != steps) continue;
-    const double c = estimate3(g, t[i], sms);
+    const double c = estimate3(g, t[i], dt == QW_C64 ? 8 : 16, sms);
     if (best < 0 || c < bc) {
       best = i;
       bc = c;
