@@ -37,9 +37,11 @@ WORKLOAD = {"name": "bcc_N512_stencil_c64", "dim": 3, "N": 512, "mass": 0.1, "si
 FALLBACK_HBM_GBS = 6800.0
 # DRAM bytes (read + write) per launch of a stencil kernel from one ncu capture of it at BCC N=384
 # (14,155,776 sites), per site.  Traffic grows in proportion to the sites, so bench.py reports
-# sites x this figure; kernels without a capture get null.
+# sites x this figure; kernels without a capture get null.  (The marching kernel's figure is from a four-step launch
+# at N=512, the launch it makes there.)
 NCU_TRAFFIC_BYTES_PER_SITE = {"step3d_c64_tma_kernel": (469785600 + 409331968) / 14155776,
-                              "step3d_c64_tma2_kernel": (476398848 + 408239360) / 14155776}
+                              "step3d_c64_tma2_kernel": (476398848 + 408239360) / 14155776,
+                              "march3d_kernel": (1431830000 + 1030636000) / 33554432}
 
 
 def parse():
@@ -238,9 +240,14 @@ def run_ours(args, rank, world, local):
     plan = qb.Plan(dim, N, W["mass"], "c64")
     if args.stencil:
         plan.set_stencil(args.stencil)
-    kernel_name = {1: "step3d_kernel<float>", 2: "step3d_c64_vec_kernel", 3: "step3d_c64_tma_kernel",
+    kernel_name = {1: "march3d_kernel", 2: "step3d_c64_vec_kernel", 3: "step3d_c64_tma_kernel",
                    4: "step3d_c64_tma2_kernel"}[plan.stencil]
-    fused = 2 if plan.stencil == 4 else 1   # steps per stencil launch
+    # stencil launches of a step.  The marching kernels take up to four steps each: 100 steps at N = 512 run as
+    # four launches of three steps and 22 of four; other workloads count the fewest possible.
+    stencil_launches = -(-S // {1: 4, 4: 2}.get(plan.stencil, 1))
+    if plan.stencil == 1 and (N, S) == (512, 100):
+        stencil_launches = 26
+    fused = S / stencil_launches   # steps per stencil launch, on average
     a = inputs.gaussian_packet(dim, N, (N / 2,) * 3, W["sigma"], W["k0"], [0.5, 0.5j, 0.5, -0.5j])
     host = torch.from_numpy(a.astype(np.complex64)).pin_memory()
     psi = host.to(dev)
@@ -280,10 +287,9 @@ def run_ours(args, rank, world, local):
     stencil_ms = sum(e[0].elapsed_time(e[1]) for e in ev)
     ms = max_over_ranks(total_ms, world, dev)
     value = job_value(sites, S, args.steps, world, ms)
-    # stencil launches (S / fused, S even) + the observables: the z FFT pass (which also takes norm
+    # stencil launches + the observables: the z FFT pass (which also takes norm
     # and <x>) and its two-stage fold, the y pass, the x-pass weights kernel (the x transform happens
     # inside it) and its two-stage fold
-    stencil_launches = (S + fused - 1) // fused
     launches_per_step = stencil_launches + 3 + 1 + 3
 
     # end-to-end through the C ABI with host buffers: qw_run_host copies every step's field
@@ -353,7 +359,8 @@ def run_ours(args, rank, world, local):
                      "traffic": (NCU_TRAFFIC_BYTES_PER_SITE[kernel_name] * sites
                                  if kernel_name in NCU_TRAFFIC_BYTES_PER_SITE else None),
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of this kernel at "
-                                       "BCC N=384, scaled by sites (profiles/%s_bcc_N384.txt)" % kernel_name,
+                                       "one BCC launch, scaled by sites (profiles/%s_bcc_N%d.txt)"
+                                       % (kernel_name, 512 if plan.stencil == 1 else 384),
                      "kernel": kernel_name, "peak_kind": peak_kind,
                      "algorithmic_bytes_per_launch": alg_bytes,
                      "steps_per_launch": fused,

@@ -57,7 +57,9 @@ typedef enum {
 typedef enum { QW_C64 = 0, QW_C128 = 1 } qw_dtype;
 
 /* Kernel used by qw_step.  All variants compute the same update; they differ in
- * data movement.  PLAIN: any geometry and dtype, one thread per site.  VEC: BCC,
+ * data movement.  PLAIN: any geometry and dtype; several steps per launch with the
+ * field's levels in registers (chains, complex64 square lattices, BCC boxes), one
+ * thread per site otherwise.  VEC: BCC,
  * complex64, N/2 % 64 == 0; two cells per thread, 16-byte loads.  TMA: BCC,
  * complex64, N/2 % 64 == 0; z-marching CTAs with TMA-staged shared-memory tiles.
  * TMA2: as TMA with two steps fused per pass over HBM (temporal fusion; an odd
