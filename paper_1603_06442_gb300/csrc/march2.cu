@@ -2,12 +2,12 @@
 // qw_march2.cuh, the split of a field over its warps, and (for the BCC boxes too) the mix of launches
 // that makes a number of steps.
 //
-// complex64, one GB300: N = 2998, 150 steps: 7.03 ms against 15.3 ms of one thread per site and one
-// pass per step; G site-steps/s of the kernel: N = 8192: 263 (four steps a pass) against 94.  It is bound by the FP32 pipe
+// complex64, one GB300: N = 2998, 150 steps: 5.8 ms against 15.3 ms of one thread per site and one
+// pass per step; G site-steps/s: N = 8192: 245 (four steps a pass) against 94.  It is bound by the FP32 pipe
 // and issue (IPC 0.64; 41 additions, 16 packed mass operations and 4 shuffles a site-step), then by
-// the halo of 8 in 64 columns; HBM is at 40%.  Measured slower: rows handed from level to level one
-// row late, so that the levels are independent (253 at N = 8192), and the sums in packed additions
-// (244: fewer instructions, the same pipe).
+// the halo of 8 in 64 columns; HBM is at 40%.  Measured slower (the kernel alone makes 263 at
+// N = 8192): rows handed from level to level one row late, so that the levels are independent (253),
+// and the sums in packed additions (244: fewer instructions, the same pipe).
 // One step, and complex128 (64 FP64 instructions a site-step on the FP64 pipe, where a recomputed
 // halo costs as much as shared sums save: 523 against 539 us at N = 2048), stay with one thread per
 // site (stencil.cu).
@@ -46,9 +46,11 @@ March2 geometry2(int64_t N, const Strip2& s, int sms, double* us) {
     const int rows = (p.N + c - 1) / c, chunks = (p.N + rows - 1) / rows;
     const int64_t items = (int64_t)p.ntx * chunks;
     const int64_t waves = (items + full - 1) / full;
-    // rows of the SM with most warps: full waves, or a part of one between the two measured ends
+    // time a row of the SM with most warps: of full waves, or of a part of one.  Half the warps take two
+    // thirds of the time, not half: with one warp a scheduler nothing fills its waits (a proportional
+    // share left N = 2998 and 8192 half empty: 192 and 198 against 232 and 245 G site-steps/s)
     const double share = waves > 1 ? 1.0 : (double)((items + sms - 1) / sms) / (s.ctas * s.nw);
-    const double t = waves * (rows + 2 * s.t) * std::max(s.own, s.full * share);
+    const double t = waves * (rows + 2 * s.t) * std::max(s.own, s.full * (0.33 + 0.67 * share));
     if (best < 0 || t < best) {
       best = t;
       p.rows = rows;
