@@ -30,9 +30,10 @@ __device__ __forceinline__ double2 shfl_c(double2 v, int src) {
 
 // steps <= 16 K - 1.  Global accesses are element wise and coalesced; the window is turned between
 // that order and the lanes' K consecutive sites in shared memory (rows of K padded to K + 1).
+// Plain loads: the launch before may still be writing `in` while this grid starts (launch_overlapped).
 template <typename R, int K>
 __global__ void __launch_bounds__(32 * kWarps1)
-    march1d_kernel(const typename CplxOf<R>::T* __restrict__ in, typename CplxOf<R>::T* __restrict__ out, int64_t N,
+    march1d_kernel(const typename CplxOf<R>::T* in, typename CplxOf<R>::T* out, int64_t N,
                    int steps, int64_t windows, typename CoefOf<R>::T cf) {
   using C = typename CplxOf<R>::T;
   constexpr int W = 32 * K;
@@ -49,7 +50,7 @@ __global__ void __launch_bounds__(32 * kWarps1)
 #pragma unroll
     for (int q = 0; q < 2; ++q)
 #pragma unroll
-      for (int i = 0; i < K; ++i) p[q][i] = __ldg(in + q * N + s0 + i * 32 + lane);
+      for (int i = 0; i < K; ++i) p[q][i] = in[q * N + s0 + i * 32 + lane];
   } else {  // around the chain's end, for a window longer than the chain more than once
     if (s0 < 0) s0 += N;
     if (s0 < 0) s0 = N - 1 - (-s0 - 1) % N;
@@ -57,8 +58,8 @@ __global__ void __launch_bounds__(32 * kWarps1)
     for (int i = 0; i < K; ++i) {
       int64_t s = s0 + i * 32 + lane;
       if (s >= N) s = N >= W ? s - N : s % N;
-      p[0][i] = __ldg(in + s);
-      p[1][i] = __ldg(in + N + s);
+      p[0][i] = in[s];
+      p[1][i] = in[N + s];
     }
   }
 #pragma unroll

@@ -55,8 +55,11 @@ inline int resident_blocks(K* kernel, int threads, int smem = 0) {
 
 // Launch that may start while the stream's previous kernel drains (programmatic stream
 // serialisation): the kernel calls grid_wait() before its first access to global memory, which
-// returns when every earlier kernel of the stream has completed and its writes are visible.  A
-// dependent launch then costs 1.4 us instead of 2.1 to 4.1 on GB300 (a kernel's end is otherwise
+// returns when every earlier kernel of the stream has completed and its writes are visible.  What the
+// kernel before writes is then read with plain loads or cp.async only: the non-coherent path (__ldg,
+// const __restrict__) is for data that nothing writes in the kernel's whole lifetime, which here begins
+// before grid_wait(), and grid_wait() does not hold such a load back.
+// A dependent launch then costs 1.4 us instead of 2.1 to 4.1 on GB300 (a kernel's end is otherwise
 // noticed at intervals of about 2 us).  overlap = false is a plain launch: for a kernel other than
 // the previous one.  An SM changes its split of L1 and shared memory only when it is empty, and a
 // kernel that overlaps another one's end keeps that one's split, also for the launches after it:
