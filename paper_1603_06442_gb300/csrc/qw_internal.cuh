@@ -65,10 +65,10 @@ inline int resident_blocks(K* kernel, int threads, int smem = 0) {
 // kernel that overlaps another one's end keeps that one's split, also for the launches after it:
 // a third slower where it leaves less L1 for the loads in flight (square lattice, N = 2998).
 template <typename... P, typename... A>
-inline qw_status launch_overlapped(void (*kernel)(P...), unsigned grid, unsigned block, int smem, bool overlap,
+inline qw_status launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned block, int smem, bool overlap,
                                    cudaStream_t st, A... args) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(grid);
+  cfg.gridDim = grid;
   cfg.blockDim = dim3(block);
   cfg.dynamicSmemBytes = (size_t)smem;
   cfg.stream = st;

@@ -183,11 +183,17 @@ __device__ __forceinline__ void coset_phase(int64_t fsum, int64_t M, T& ar, T& a
   }
 }
 
-// Position of the thread in a 3D launch over (nx, ny, nz); false when outside.
+// Position of the thread in a launch of point_grid (spectral.cu); false when outside.  A grid over
+// rows has (y, z) in its indices, and a chain has x only: neither divides.  A grid of one row over a box
+// counts its positions, x fastest.
 __device__ __forceinline__ bool grid_pos(const AxesDev& a, int64_t& x, int64_t& y, int64_t& z) {
-  // one thread per position of the box, x fastest: a grid over rows would leave most of a CTA idle
-  // on boxes narrower than it (a box of 81^3 cells used 81 of 256 threads)
   const int64_t idx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (gridDim.y > 1 || a.len[1] == 1) {
+    x = idx;
+    y = blockIdx.y;
+    z = blockIdx.z;
+    return x < a.len[0];
+  }
   const int64_t total = a.len[0] * a.len[1] * a.len[2];
   if (idx >= total) return false;
   if (total <= 0x7fffffff) {  // 32-bit index arithmetic

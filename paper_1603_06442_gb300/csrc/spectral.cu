@@ -142,9 +142,9 @@ __global__ void omega_dd_kernel(int dim, AxesDev a, double m, const double2* __r
 template <typename T>
 __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t count, Mass ms,
                                                      const double* __restrict__ omega, TimeArg ta, T scale,
-                                                     typename Cx2<T>::t* __restrict__ data) {
+                                                     typename Cx2<T>::t* __restrict__ data, int overlap) {
   using V = typename Cx2<T>::t;
-  grid_wait();
+  if (overlap) grid_wait();
   int64_t x, y, z;
   if (grid_pos(a, x, y, z)) {
     const int64_t idx = (z * a.len[1] + y) * a.len[0] + x;
@@ -162,8 +162,9 @@ __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t
 
 template <typename T>
 __global__ void __launch_bounds__(256) fw_kernel(int dim, AxesDev a, int64_t count, Mass ms, T scale,
-                                                 typename Cx2<T>::t* __restrict__ data) {
+                                                 typename Cx2<T>::t* __restrict__ data, int overlap) {
   using V = typename Cx2<T>::t;
+  if (overlap) grid_wait();
   int64_t x, y, z;
   if (!grid_pos(a, x, y, z)) return;
   const int64_t idx = (z * a.len[1] + y) * a.len[0] + x;
@@ -328,7 +329,16 @@ constexpr int kPointThreads = 256, kPointSmall = 128;
 static int point_threads(const Geometry& g, qw_dtype dt) {
   return dt == QW_C128 && g.vol <= 152 * kPointThreads ? kPointSmall : kPointThreads;
 }
-static unsigned point_grid(const Geometry& g, int threads) { return (unsigned)((g.vol + threads - 1) / threads); }
+// Rows of CTAs where they fill (an eighth idle at most) and fit the grid, else the box's positions in
+// one row: a box of 81^3 cells uses 81 of a row's 256 threads.  The positions' divisions cost a long
+// row 2 to 4% (Foldy-Wouthuysen transform, chain of 2^24: 1062 against 1023 us; square lattice
+// N = 4096: 2091 against 2053 us).
+static dim3 point_grid(const Geometry& g, int threads) {
+  const int64_t row = (g.nx + threads - 1) / threads;
+  if (g.ny * g.nz == 1 || (8 * g.nx >= 7 * row * threads && g.ny <= 65535 && g.nz <= 65535))
+    return dim3((unsigned)row, (unsigned)g.ny, (unsigned)g.nz);
+  return dim3((unsigned)((g.vol + threads - 1) / threads));
+}
 
 // complex128 plans: the double-double omega table (16 bytes per stored wave vector).  The
 // per-axis and anchor tables it needs live in one temporary buffer (synchronous).
@@ -386,9 +396,9 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
   if (dt == QW_C64)
     return launch_overlapped(evolve_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
                              count, make_mass(n, m), omega, make_time(t), (float)inv,
-                             static_cast<float2*>(psi_hat));
+                             static_cast<float2*>(psi_hat), overlap);
   return launch_overlapped(evolve_kernel<double>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
-                           count, make_mass(n, m), omega, make_time(t), inv, static_cast<double2*>(psi_hat));
+                           count, make_mass(n, m), omega, make_time(t), inv, static_cast<double2*>(psi_hat), overlap);
 }
 
 template <int DIM>
@@ -416,14 +426,13 @@ qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt
                               cudaStream_t st) {
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
+  const int threads = point_threads(g, dt);
+  const bool overlap = small_field(g, dt);
   if (dt == QW_C64)
-    fw_kernel<float><<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), (float)inv,
-                                               static_cast<float2*>(psi_hat));
-  else
-    fw_kernel<double><<<point_grid(g, kPointThreads), kPointThreads, 0, st>>>(g.dim, to_dev(ax), count, make_mass(n, m), inv,
-                                                static_cast<double2*>(psi_hat));
-  QW_CHECK_LAUNCH("Foldy-Wouthuysen launch");
-  return QW_OK;
+    return launch_overlapped(fw_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax), count,
+                             make_mass(n, m), (float)inv, static_cast<float2*>(psi_hat), overlap);
+  return launch_overlapped(fw_kernel<double>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax), count,
+                           make_mass(n, m), inv, static_cast<double2*>(psi_hat), overlap);
 }
 
 bool fused_x_supported(const Geometry& g, const FftPlan& f, qw_dtype dt) {
