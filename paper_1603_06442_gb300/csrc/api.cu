@@ -68,6 +68,17 @@ int resident_blocks_once(const void* func, int threads, int smem) {
   return known[key] = per_sm * sms;
 }
 
+int sm_count() {
+  constexpr int kDevices = 64;
+  static std::atomic<int> known[kDevices];
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 0;
+  if (dev < kDevices && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
+  if (dev < kDevices) known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
 static std::atomic<bool> g_poison{false};
 bool debug_poison() { return g_poison.load(std::memory_order_relaxed); }
 

@@ -172,12 +172,10 @@ __global__ void __launch_bounds__(256) fft_pass_kernel(typename Cx<T>::t* __rest
   }
 }
 
-// Passes over at most 4 MB (as small_field) are launched to overlap; the larger ones skip the wait, which
-// cost 1 us a pass (BCC, N = 512 evolution: 2286 us with it, 2280 without).
-__host__ __device__ inline bool pass_overlaps(const FftPass& p, int64_t elem) { return p.O * p.S * p.L * elem <= (4 << 20); }
-
 // MOM (forward strided passes of the observables): the position moments of the loaded lines
 // (FftMoments) are summed before the transform, one partial per CTA.
+// overlap: overlap_mode (passes over at most 4 MB; the larger ones skip the wait, which cost 1 us a pass:
+// BCC, N = 512 evolution 2286 us with it, 2280 without).
 // NT: threads per CTA (256, or 128 for FP64 lines too few to fill the SMs: an FP64 instruction holds a
 // quarter of an SM for 64 clocks a warp, so four warps an SM finish in half the time of eight).
 template <typename T, bool INV, int R1, int R2, bool CONTIG, bool MOM = false, int NT = 256>
@@ -185,7 +183,7 @@ __global__ void __launch_bounds__(NT) fft2f_kernel(typename Cx<T>::t* data, cons
                                                     const typename Cx<T>::t* __restrict__ tw_line,
                                                     const typename Cx<T>::t* __restrict__ tw_hi,
                                                     const typename Cx<T>::t* __restrict__ tw_lo,
-                                                    FftMoments mom = FftMoments{}) {
+                                                    FftMoments mom = FftMoments{}, int overlap = 0) {
   using V = typename Cx<T>::t;
   constexpr int L = R1 * R2;
   constexpr int TPL = R1 > R2 ? R1 : R2;  // threads per line
@@ -194,7 +192,7 @@ __global__ void __launch_bounds__(NT) fft2f_kernel(typename Cx<T>::t* data, cons
   extern __shared__ __align__(16) unsigned char f2_smem[];
   V* sm = reinterpret_cast<V*>(f2_smem);
   const int tid = threadIdx.x;
-  if (pass_overlaps(p, sizeof(V))) grid_wait();
+  if (overlap & kAwait) grid_await();
   const int64_t S = p.S;
   const int64_t nlines = p.O * S;
   const int64_t l0 = (int64_t)blockIdx.x * C;
@@ -297,6 +295,7 @@ __global__ void __launch_bounds__(NT) fft2f_kernel(typename Cx<T>::t* data, cons
       }
     }
   }
+  if (overlap & kRelease) grid_release();
   // ---- store
   if (CONTIG) {
     constexpr int NE = (C * L + NT - 1) / NT;
@@ -322,7 +321,7 @@ __global__ void __launch_bounds__(NT) fft2f_kernel(typename Cx<T>::t* data, cons
 }
 
 template <typename T, bool INV, int R1, int R2, int NT>
-static qw_status launch_2f_nt(const FftPass& p, void* data, const void* src, bool overlap, cudaStream_t st) {
+static qw_status launch_2f_nt(const FftPass& p, void* data, const void* src, cudaStream_t st) {
   using V = typename Cx<T>::t;
   constexpr int L = R1 * R2, TPL = R1 > R2 ? R1 : R2, C = NT / TPL;
   const size_t smem = (size_t)L * ((C % 2 == 0) ? C + 1 : C) * sizeof(V);
@@ -335,19 +334,19 @@ static qw_status launch_2f_nt(const FftPass& p, void* data, const void* src, boo
   auto* kernel = p.S == 1 ? fft2f_kernel<T, INV, R1, R2, true, false, NT> : fft2f_kernel<T, INV, R1, R2, false, false, NT>;
   const qw_status sa = smem_attr(kernel, (int)smem);
   if (sa != QW_OK) return sa;
+  const int overlap = overlap_mode(small_bytes(nlines * L * (int64_t)sizeof(V)), sizeof(T) == 8, grid);
   return launch_overlapped(kernel, (unsigned)grid, NT, (int)smem, overlap, st, static_cast<V*>(data),
                            static_cast<const V*>(src), p, static_cast<const V*>(p.tw_line),
-                           static_cast<const V*>(p.tw_hi), static_cast<const V*>(p.tw_lo), FftMoments{});
+                           static_cast<const V*>(p.tw_hi), static_cast<const V*>(p.tw_lo), FftMoments{}, overlap);
 }
 
 template <typename T, bool INV, int R1, int R2>
 static qw_status launch_2f(const FftPass& p, void* data, const void* src, cudaStream_t st) {
   constexpr int TPL = R1 > R2 ? R1 : R2;
   const int64_t nlines = p.O * p.S;
-  const bool overlap = pass_overlaps(p, sizeof(typename Cx<T>::t));
   if constexpr (sizeof(T) == 8)
-    if (nlines <= 152 * (256 / TPL)) return launch_2f_nt<T, INV, R1, R2, 128>(p, data, src, overlap, st);
-  return launch_2f_nt<T, INV, R1, R2, 256>(p, data, src, overlap, st);
+    if (nlines <= 152 * (256 / TPL)) return launch_2f_nt<T, INV, R1, R2, 128>(p, data, src, st);
+  return launch_2f_nt<T, INV, R1, R2, 256>(p, data, src, st);
 }
 
 // f(R1, R2) (as integral constants) for a register length L >= 64; false for other lengths.

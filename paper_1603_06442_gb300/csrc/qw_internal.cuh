@@ -35,6 +35,7 @@ inline qw_status smem_attr(K* kernel, int bytes) {
   return smem_attr_once(reinterpret_cast<const void*>(kernel), bytes);
 }
 // Blocks of a kernel resident on the current device at once (0 if the query fails).
+int sm_count();  // multiprocessors of the current device (0 on error)
 int resident_blocks_once(const void* func, int threads, int smem);
 template <typename K>
 inline int resident_blocks(K* kernel, int threads, int smem = 0) {
@@ -81,10 +82,15 @@ inline qw_status launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned blo
   return QW_OK;
 }
 #ifdef __CUDACC__
+__device__ __forceinline__ void grid_await() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+// The next launch may follow: its CTAs are placed once all of this grid's have come here or are done.
+__device__ __forceinline__ void grid_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// Both at once: the next launch's CTAs take whatever room there is from the start.  Where they are bound
+// by a pipe of the SM and there is room for several, they crowd the SMs that this grid leaves empty; such
+// kernels release after their arithmetic instead.
 __device__ __forceinline__ void grid_wait() {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  // every CTA of this grid is resident or done once all have come here: the next launch may follow
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  grid_await();
+  grid_release();
 }
 #endif
 
@@ -122,7 +128,16 @@ bool make_geometry(int dim, int64_t N, Geometry* g);
 
 // Fields whose kernels run a few us each: their passes are launched to overlap (launch_overlapped;
 // the split of L1 and shared memory does not matter where most of an SM is idle).
-inline bool small_field(const Geometry& g, qw_dtype dt) { return g.elems * (dt == QW_C64 ? 8 : 16) <= (4 << 20); }
+inline bool small_bytes(int64_t bytes) { return bytes <= (4 << 20); }
+inline bool small_field(const Geometry& g, qw_dtype dt) { return small_bytes(g.elems * (dt == QW_C64 ? 8 : 16)); }
+// How such a launch overlaps (a kernel argument): it awaits the launch before, and lets the next one follow
+// after its arithmetic.  In FP64 only where both launches' CTAs have SMs of their own, else when it is done:
+// a CTA placed beside another one while SMs are about to fall idle takes twice as long (evolution of a chain
+// of 2^17 sites in complex128: 186 us where every launch let the next one in at its start, 123 us where none did).
+constexpr int kAwait = 1, kRelease = 2;
+inline int overlap_mode(bool small, bool fp64, int64_t ctas) {
+  return !small ? 0 : (fp64 && 2 * ctas > sm_count()) ? kAwait : kAwait | kRelease;
+}
 
 // Fields need only element alignment (8 bytes in complex64); kernels that move 16-byte
 // vectors are chosen only for fields that are 16-byte aligned.

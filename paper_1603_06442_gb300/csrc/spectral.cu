@@ -144,7 +144,7 @@ __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t
                                                      const double* __restrict__ omega, TimeArg ta, T scale,
                                                      typename Cx2<T>::t* __restrict__ data, int overlap) {
   using V = typename Cx2<T>::t;
-  if (overlap) grid_wait();
+  if (overlap & kAwait) grid_await();
   int64_t x, y, z;
   if (grid_pos(a, x, y, z)) {
     const int64_t idx = (z * a.len[1] + y) * a.len[0] + x;
@@ -154,6 +154,7 @@ __global__ void __launch_bounds__(256) evolve_kernel(int dim, AxesDev a, int64_t
     for (int q = 0; q < 8; ++q)
       if (q < P) v[q] = data[q * count + idx];
     evolve_point<T>(dim, a, x, y, z, idx, ms, omega, ta, scale, v);
+    if (overlap & kRelease) grid_release();
 #pragma unroll
     for (int q = 0; q < 8; ++q)
       if (q < P) data[q * count + idx] = v[q];
@@ -164,7 +165,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) fw_kernel(int dim, AxesDev a, int64_t count, Mass ms, T scale,
                                                  typename Cx2<T>::t* __restrict__ data, int overlap) {
   using V = typename Cx2<T>::t;
-  if (overlap) grid_wait();
+  if (overlap & kAwait) grid_await();
   int64_t x, y, z;
   if (!grid_pos(a, x, y, z)) return;
   const int64_t idx = (z * a.len[1] + y) * a.len[0] + x;
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(256) fw_kernel(int dim, AxesDev a, int64_t cou
   for (int q = 0; q < 8; ++q)
     if (q < P) v[q] = data[q * count + idx];
   fw_point<T>(dim, a, x, y, z, ms, scale, v);
+  if (overlap & kRelease) grid_release();
 #pragma unroll
   for (int q = 0; q < 8; ++q)
     if (q < P) data[q * count + idx] = v[q];
@@ -392,7 +394,7 @@ qw_status launch_evolve_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtyp
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
   const int threads = point_threads(g, dt);
-  const bool overlap = small_field(g, dt);
+  const int overlap = overlap_mode(small_field(g, dt), dt == QW_C128, g.vol / threads);
   if (dt == QW_C64)
     return launch_overlapped(evolve_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax),
                              count, make_mass(n, m), omega, make_time(t), (float)inv,
@@ -427,7 +429,7 @@ qw_status launch_fw_pointwise(const Geometry& g, const SpecAxes& ax, qw_dtype dt
   const int64_t count = kcount(g);
   const double inv = 1.0 / (double)g.vol;
   const int threads = point_threads(g, dt);
-  const bool overlap = small_field(g, dt);
+  const int overlap = overlap_mode(small_field(g, dt), dt == QW_C128, g.vol / threads);
   if (dt == QW_C64)
     return launch_overlapped(fw_kernel<float>, point_grid(g, threads), threads, 0, overlap, st, g.dim, to_dev(ax), count,
                              make_mass(n, m), (float)inv, static_cast<float2*>(psi_hat), overlap);

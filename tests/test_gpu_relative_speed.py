@@ -1,0 +1,42 @@
+"""Calls that must not fall behind another call on the same work: ratios of best-of-many device times, with bounds
+between what the library reaches and what the faults named here cost."""
+
+import pytest
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.fixture(scope="module")
+def qb(qwlib):
+    from paper_1603_06442_gb300 import binding
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    return binding
+
+
+def best_ms(fn, calls=10, repeats=7):
+    fn()
+    best = float("inf")
+    for _ in range(repeats):
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(calls):
+            fn()
+        b.record()
+        b.synchronize()
+        best = min(best, a.elapsed_time(b) / calls)
+    return best
+
+
+def test_overlapped_fp64_passes_do_not_crowd_sms(qb):
+    """Half the chain takes 0.55 of the time; 0.84 where each launch's CTAs are placed while the one before runs."""
+    ms = []
+    for N in (1 << 17, 1 << 18):
+        plan = qb.Plan(1, N, 0.1, "c128")
+        x = torch.zeros(plan.elems, dtype=torch.complex128, device="cuda")
+        plan.prepare_spectral()
+        ms.append(best_ms(lambda: plan.evolve_spectral(x, 1000)))
+        plan.close()
+    assert ms[0] < 0.7 * ms[1], ms
