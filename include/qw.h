@@ -311,12 +311,13 @@ qw_status qw_batch_destroy(qw_batch batch);
 
 /* How a batch cuts its walks into work items.  A round advances one tile of a walk
  * by `depth` steps (its fusion depth, per lattice dimension):
- *   depth 1: where no walk of the batch has a larger depth, walks of the square
- *            lattice and BCC boxes advance by four and three steps per round, the
- *            steps between held in registers (the tiles are the kernel's own; the
- *            steps left over take a round each); chains, and every depth-1 walk of
- *            a batch with fused ones, update every site from global memory; tiles
- *            are whole x rows (x segments on the chain) of about tile_sites sites;
+ *   depth 1: every site updated from global memory; tiles are whole x rows (x
+ *            segments on the chain) of about tile_sites sites.  Where no walk of the
+ *            batch has a larger depth and the batch is large enough for it to pay
+ *            (estimated per tiling), walks of the square lattice and BCC boxes instead
+ *            advance by four and three steps per round, the steps between held in
+ *            registers (the tiles are the kernel's own; steps left over take a round
+ *            each);
  *   depth 2..4: temporal fusion; the tile is a box of box[dim-1] = (x, y, z)
  *            cells (both cosets on the BCC lattice; unused axes ignored), which
  *            is read with a halo of `depth` cells per side (depth/2 rounded up on

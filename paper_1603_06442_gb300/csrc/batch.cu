@@ -8,10 +8,10 @@
 // (r + 1) % 2; when the number of stepping rounds is odd a last round copies
 // the result back into the caller's field.  The fusion depth T_w is set per
 // lattice dimension:
-//   * T = 1, when no walk of the batch is fused: marching rounds of the square lattice (four
-//     steps) and BCC boxes (three) with the steps between held in registers (qw_march.cuh,
-//     qw_march2.cuh), the steps left over one per round.  The 256-walk mix on one GB300: 132 ms
-//     against 307 ms of per-site rounds (161 against 69 G site-steps/s);
+//   * T = 1, when no walk of the batch is fused and the batch is large (march_pays): marching rounds
+//     of the square lattice (four steps) and BCC boxes (three) with the steps between held in
+//     registers (qw_march.cuh, qw_march2.cuh), the steps left over one per round.  The 256-walk mix
+//     on one GB300: 132 ms against 307 ms of per-site rounds (161 against 69 G site-steps/s);
 //   * T = 1 else, and on the chain: each cell is updated from global memory (the per-site update);
 //   * T >= 2 (temporal fusion): the tile and a halo of H cells per side (H = T on
 //     the chain and the square lattice, ceil(T/2) on the BCC lattice, where one
@@ -93,13 +93,23 @@ struct BatchDebug {
 };
 
 constexpr long long kBatchSpin = 1ll << 24;
-// Marching launches (no walk fused in shared memory): four warps, two CTAs per SM.  A square-lattice
+// What a launch runs: per-site rounds only, marching rounds (and per-site ones for chains and the steps
+// left over), or fused rounds in shared memory (and per-site ones for walks of depth 1).
+enum BatchKind { kPlainBatch, kMarchBatch, kFusedBatch };
+// Per-site launches live by the loads in flight: 1024 threads per SM at 64 registers, no spills (6 and 3
+// CTAs, and cells taken two at a time, measured 2-15% slower on the uneven 256-walk mix).
+constexpr int kBatchThreads = 256, kBatchMinBlocks = 4;
+// Marching launches: four warps, two CTAs per SM.  A square-lattice
 // item is a strip of kCols columns and four warps' rows, kT2 steps; a BCC item a tile of
 // tile3_geo(M, 1, kRows3, kT3, 4) and a chunk of layers, kT3 steps.
 constexpr int kMarchThreads = 128, kT2 = 4, kCols = 64 - 2 * kT2, kT3 = 3, kRows3 = 3;
 constexpr int kMarchSmem = march2_smem<2, 4>() > march3_smem<float, 1, kRows3, 4>() ? march2_smem<2, 4>()
                                                                                    : march3_smem<float, 1, kRows3, 4>();
 constexpr int kFusedThreads = 256;   // launches with fused rounds (512 measured slower: 172 vs 232 G on the chain)
+constexpr int batch_threads(int kind) {
+  return kind == kMarchBatch ? kMarchThreads : kind == kFusedBatch ? kFusedThreads : kBatchThreads;
+}
+constexpr int batch_blocks(int kind) { return kind == kMarchBatch ? 2 : kind == kFusedBatch ? 3 : kBatchMinBlocks; }
 
 // Largest i in [0, n) with a[i] <= v (a ascending, a[0] <= v), searched by the 32 lanes
 // of a warp together: each round cuts the range into 32 slices and keeps the last
@@ -353,15 +363,13 @@ __device__ __forceinline__ void march_round(const BatchWalk& W, const int (&t3)[
   }
 }
 
-// FUSED = false: walks of the square lattice and BCC boxes run marching rounds, chains per-site
-// rounds; FUSED = true: walks of depth >= 2 run fused rounds in dynamic shared memory, the others
-// per-site rounds.
-template <bool FUSED>
-__global__ void __launch_bounds__(FUSED ? kFusedThreads : kMarchThreads, FUSED ? 3 : 2)
+template <int KIND>
+__global__ void __launch_bounds__(batch_threads(KIND), batch_blocks(KIND))
     batch_kernel(const BatchWalk* __restrict__ walks, const BatchGroup* __restrict__ groups,
                  const int64_t* __restrict__ group_item0, int ngroups, const int64_t* __restrict__ tile_prefix,
                  const int64_t* __restrict__ round_prefix, int64_t total_items, unsigned int* __restrict__ done,
                  BatchCtl* __restrict__ ctl, BatchDebug dbg) {
+  constexpr int NT = batch_threads(KIND);
   extern __shared__ __align__(16) float2 smem_dyn[];
   __shared__ int64_t s_next, s_round;
   __shared__ int s_abort, s_walk, s_tile;
@@ -458,9 +466,8 @@ __global__ void __launch_bounds__(FUSED ? kFusedThreads : kMarchThreads, FUSED ?
     if (s < W.nstep) {
       const float2* in = (s & 1) ? b1 : b0;
       float2* out = (s & 1) ? b0 : b1;
-      constexpr int NT = FUSED ? kFusedThreads : kMarchThreads;
       bool done_round = false;
-      if constexpr (FUSED) {
+      if constexpr (KIND == kFusedBatch) {
         if (W.depth > 1) {
           const int steps = (int)min((int64_t)W.depth, W.t - s * W.depth);
           const int P = (W.ncos * W.ncomp) * (W.ext[0] + 2 * W.halo) * (W.dim >= 2 ? W.ext[1] + 2 * W.halo : 1) *
@@ -468,13 +475,13 @@ __global__ void __launch_bounds__(FUSED ? kFusedThreads : kMarchThreads, FUSED ?
           fused_round<NT>(W, t3, steps, in, out, smem_dyn, smem_dyn + P);
           done_round = true;
         }
-      } else if (s < W.nfull) {
+      } else if (KIND == kMarchBatch && s < W.nfull) {
         march_round(W, t3, in, out, reinterpret_cast<unsigned char*>(smem_dyn));
         done_round = true;
       }
       if (!done_round) plain_round<NT>(W, t3, false, in, out);
     } else {
-      plain_round<FUSED ? kFusedThreads : kMarchThreads>(W, t3, true, b1, b0);  // copy round: the result sits in buf[1]
+      plain_round<NT>(W, t3, true, b1, b0);  // copy round: the result sits in buf[1]
     }
     __syncthreads();
     if (tid == 0 && W.tile_base + tile != dbg.stall_tile) {
@@ -521,8 +528,8 @@ struct qw_batch_s {
   int ngroups = 0;
   int64_t total_items = 0;
   qw_batch_tiling tiling;
-  bool fused = false;      // some walk has depth >= 2: the fused kernel runs the launch
-  size_t smem = 0;         // its dynamic shared memory
+  int kind = kPlainBatch;  // BatchKind
+  size_t smem = 0;         // dynamic shared memory of the launch
   int grid = 0;
   BatchDebug dbg = {-1, kBatchSpin};
   int stall_walk = -1;     // caller's index of the walk whose first tile is stalled
@@ -712,6 +719,57 @@ qw_status launch_step_fused(const Geometry& g, int depth, const int* box, int st
   return QW_OK;
 }
 
+static decltype(&batch_kernel<kPlainBatch>) batch_kernel_of(int kind) {
+  return kind == kMarchBatch ? batch_kernel<kMarchBatch>
+         : kind == kFusedBatch ? batch_kernel<kFusedBatch> : batch_kernel<kPlainBatch>;
+}
+
+// Estimated us of a group's walks W in a launch without fused rounds.  Walks share the SMs (work: sites at
+// the rate of the rounds, marching items on two CTAs per SM) but a walk's rounds follow one another (chain:
+// the longest walk on its own); the two are joined as sides of a right angle.  Constants fitted to 228
+// batches of 1 to 200 walks of every lattice, t = 1 to 600, run both ways on one GB300 (rms 12 and 15%).
+static double group_us(const std::vector<BatchWalk>& walks, bool march) {
+  // site-steps per us with the SMs full, by lattice; us of a round, and per cell of a thread
+  const double rate[2][3] = {{117e3, 82e3, 60e3}, {48e3, 36e3, 27e3}};
+  const double cell[2][3] = {{0.48, 0.74, 1.1}, {0.46, 0.46, 0.46}};
+  const double round[2] = {1.5, 0.85}, copy[2] = {1.3, 1.96};  // a copy round, in steps
+  // us per row (half-layer) of a marching item: of the launch with the SMs full, of an item on its own
+  const double full = 0.95 / (2.0 * sm_count()), alone[3] = {0.0, 0.70, 0.95};
+  const int m = march ? 1 : 0, threads = march ? kMarchThreads : kBatchThreads;
+  double work = 0.0, chain = 0.0;
+  for (const BatchWalk& W : walks) {
+    const double sites = (double)W.vol * W.ncos;
+    const int cells = (W.ncos * W.ext[0] * W.ext[1] * W.ext[2] + threads - 1) / threads;
+    const double single = (double)(W.nstep - W.nfull) + copy[m] * (double)(W.rounds - W.nstep);  // per-site rounds
+    const int rows = W.dim == 2 ? W.ext[1] / 4 + 2 * kT2 : 2 * W.ext[2] + 2 * kT3;
+    work += sites * single / rate[m][W.dim - 1] + (double)W.nfull * W.ntiles * rows * full;
+    chain = std::max(chain, single * (round[m] + cells * cell[m][W.dim - 1]) + (double)W.nfull * (round[m] + rows * alone[W.dim - 1]));
+  }
+  return std::hypot(work, chain);
+}
+
+// Whether the batch's walks of the square lattice and BCC boxes march.  A marching launch holds a quarter of
+// the threads, so its per-site rounds (chains, steps left over) are slower, and its items are long, so a few
+// small walks have too few of them.  Measured per-site / marching: the 256-walk mix 307 / 132 ms, one BCC walk
+// of N = 256, 50 steps 3.3 / 1.5 ms; but one of N = 128 0.75 / 1.38 ms, 64 walks of one step each 0.23 / 0.72 ms,
+// 64 chains of 10^4 to 10^7 sites 43 / 110 ms.  Marching has to be a fifth faster by the estimates: of the
+// batches they were fitted to, 41 then march, the slowest of them 2% slower than per site.
+static bool march_pays(const std::vector<qw_walk>& desc, const std::vector<std::vector<int>>& groups,
+                       const qw_batch_tiling& tiling) {
+  double us[2] = {0.0, 0.0};
+  bool any = false;  // a marching round in the batch
+  for (int m = 0; m < 2; ++m)
+    for (const std::vector<int>& group : groups) {
+      std::vector<BatchWalk> walks;
+      for (int i : group) {
+        walks.push_back(make_walk(desc[i], nullptr, tiling, m == 1));
+        any = any || walks.back().nfull > 0;
+      }
+      us[m] += group_us(walks, m == 1);
+    }
+  return any && 1.2 * us[1] < us[0];
+}
+
 // Build the walk table, groups and prefix arrays for the current tiling, and upload them.
 static qw_status build_schedule(qw_batch_s* b) {
   free_schedule(b);
@@ -739,13 +797,13 @@ static qw_status build_schedule(qw_batch_s* b) {
   b->first_tile.assign(n, 0);
   bool fused = false;
   for (const qw_walk& d : b->desc) fused = fused || b->tiling.depth[d.dim - 1] > 1;
-  b->fused = fused;
-  b->smem = fused ? 0 : kMarchSmem;
+  b->kind = fused ? kFusedBatch : march_pays(b->desc, grp, b->tiling) ? kMarchBatch : kPlainBatch;
+  b->smem = b->kind == kMarchBatch ? kMarchSmem : 0;
   int64_t item0 = 0;
   int64_t ndone_acc = 0;
   for (auto& gw : grp) {
     std::vector<BatchWalk> gwalks;
-    for (int i : gw) gwalks.push_back(make_walk(b->desc[i], b->partners[i], b->tiling, !fused));
+    for (int i : gw) gwalks.push_back(make_walk(b->desc[i], b->partners[i], b->tiling, b->kind == kMarchBatch));
     // inside a group: most rounds first, so the walks alive at round s are a prefix
     std::vector<int> ord(gw.size());
     for (size_t k = 0; k < gw.size(); ++k) ord[k] = (int)k;
@@ -819,16 +877,10 @@ static qw_status build_schedule(qw_batch_s* b) {
   QW_CHECK_CUDA(cudaMemcpy(b->d_tiles, tiles.data(), tiles.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
   QW_CHECK_CUDA(cudaMemcpy(b->d_rounds, rounds.data(), rounds.size() * sizeof(int64_t), cudaMemcpyHostToDevice));
   int per_sm = 0, nsm = 0;
-  if (b->fused) {
-    qw_status sa = smem_attr(batch_kernel<true>, (int)b->smem);
-    if (sa != QW_OK) return sa;
-    QW_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<true>, kFusedThreads, b->smem));
-  } else {
-    qw_status sa = smem_attr(batch_kernel<false>, kMarchSmem);
-    if (sa != QW_OK) return sa;
-    QW_CHECK_CUDA(
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, batch_kernel<false>, kMarchThreads, kMarchSmem));
-  }
+  auto* kernel = batch_kernel_of(b->kind);
+  qw_status sa = smem_attr(kernel, (int)b->smem);
+  if (sa != QW_OK) return sa;
+  QW_CHECK_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, batch_threads(b->kind), b->smem));
   QW_CHECK_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, b->device));
   b->grid = std::max(1, per_sm * nsm);
   return QW_OK;
@@ -840,14 +892,9 @@ static qw_status launch_batch(qw_batch_s* b, cudaStream_t s) {
       QW_CHECK_CUDA(cudaMemsetAsync(b->partners[i], kPoisonByte, field_bytes(b->desc[i]), s));
   QW_CHECK_CUDA(cudaMemsetAsync(b->d_done, 0, std::max<int64_t>(1, b->ndone) * sizeof(unsigned int), s));
   QW_CHECK_CUDA(cudaMemsetAsync(b->d_ctl, 0, sizeof(BatchCtl), s));
-  if (b->fused)
-    batch_kernel<true><<<b->grid, kFusedThreads, b->smem, s>>>(b->d_walks, b->d_groups, b->d_group_item0,
-                                                               b->ngroups, b->d_tiles, b->d_rounds, b->total_items,
-                                                               b->d_done, b->d_ctl, b->dbg);
-  else
-    batch_kernel<false><<<b->grid, kMarchThreads, b->smem, s>>>(b->d_walks, b->d_groups, b->d_group_item0, b->ngroups,
-                                                          b->d_tiles, b->d_rounds, b->total_items, b->d_done,
-                                                          b->d_ctl, b->dbg);
+  batch_kernel_of(b->kind)<<<b->grid, batch_threads(b->kind), b->smem, s>>>(
+      b->d_walks, b->d_groups, b->d_group_item0, b->ngroups, b->d_tiles, b->d_rounds, b->total_items, b->d_done,
+      b->d_ctl, b->dbg);
   QW_CHECK_LAUNCH("batch kernel launch");
   return QW_OK;
 }

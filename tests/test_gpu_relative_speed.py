@@ -40,3 +40,15 @@ def test_overlapped_fp64_passes_do_not_crowd_sms(qb):
         ms.append(best_ms(lambda: plan.evolve_spectral(x, 1000)))
         plan.close()
     assert ms[0] < 0.7 * ms[1], ms
+
+
+def test_chains_of_a_batch_keep_their_threads(qb):
+    """A batch's rounds update a long chain at the rate of the per-site kernel in launches of one step (1.5 of its
+    time); 3.9 with a quarter of the threads per SM."""
+    N, t = 4_000_000, 40
+    x = torch.zeros((2, N), dtype=torch.complex64, device="cuda")
+    batch = qb.Batch([(1, N, 0.1, t, x)])
+    ms = best_ms(batch.run, 2)
+    batch.sync()
+    batch.close()
+    assert ms < 2.5 * best_ms(lambda: qb.qw_step_static(1, N, 0.1, "c64", x, t), 2), ms
