@@ -59,15 +59,16 @@ typedef enum { QW_C64 = 0, QW_C128 = 1 } qw_dtype;
 /* Kernel used by qw_step.  All variants compute the same update; they differ in
  * data movement.  PLAIN: any geometry and dtype; several steps per launch with the
  * field's levels in registers (chains, complex64 square lattices, BCC boxes), one
- * thread per site otherwise.  VEC: BCC,
+ * thread per site otherwise and for single steps where that is faster.  VEC: BCC,
  * complex64, N/2 % 64 == 0; two cells per thread, 16-byte loads.  TMA: BCC,
  * complex64, N/2 % 64 == 0; z-marching CTAs with TMA-staged shared-memory tiles.
  * TMA2: as TMA with two steps fused per pass over HBM (temporal fusion; an odd
  * remaining step runs as TMA).  FUSED: any lattice and size, complex64; box
  * tiles of the field with a halo loaded into shared memory, `depth` steps per
  * launch (temporal fusion of depth 2..4, tile box and depth set by
- * qw_plan_set_fusion or the autotuner).  AUTO restores the default, PLAIN, the
- * fastest measured on GB300; qw_plan_autotune measures every variant (FUSED with
+ * qw_plan_set_fusion or the autotuner).  AUTO restores the default: PLAIN, with the
+ * TMA kernels for the one- and two-step launches of large BCC boxes that they make
+ * faster (complex64, a 16-byte aligned field), the fastest measured on GB300; qw_plan_autotune measures every variant (FUSED with
  * several depths and boxes) and keeps the fastest. */
 typedef enum {
   QW_STENCIL_AUTO = 0,

@@ -160,10 +160,24 @@ bool make_geometry(int dim, int64_t N, Geometry* g) {
 }
 
 static int default_stencil(const qw_plan_s* p) {
-  // the marching kernels behind PLAIN are the fastest measured on every lattice, size and type
-  // (march1.cu, march2.cu, march3.cu); qw_plan_autotune re-measures on the device
+  // the launches behind PLAIN are the fastest measured on every lattice, size and type (march1.cu,
+  // march2.cu, march3.cu; auto_stencil adds the TMA kernels); qw_plan_autotune re-measures on the device
   (void)p;
   return QW_STENCIL_PLAIN;
+}
+
+// The launches of a run of nsteps steps of PLAIN, kept in the plan for the next run of as many (they depend on
+// the geometry and the step count alone).  table: see step_table.
+static void plan_run(qw_plan_s* p, int64_t nsteps, int table) {
+  if (p->run_steps == nsteps && p->run_table == table) return;
+  for (int64_t& k : p->run_march) k = 0;
+  p->run_chain = March1{0, 0};
+  if (march_supported(p->g, p->dtype))
+    march_schedule(p->g, p->dtype, nsteps, p->step_table[table], p->run_march);
+  else if (p->g.dim == 1)
+    p->run_chain = march1_schedule(p->g.nx, p->dtype, nsteps, p->sms);
+  p->run_steps = nsteps;
+  p->run_table = table;
 }
 
 static qw_status check_flags(qw_plan_s* p, cudaStream_t s) {
@@ -295,7 +309,14 @@ qw_status qw_plan_create(int dim, int64_t N, double mass, qw_dtype dtype, qw_pla
   p->fuse_box[0] = g.dim == 1 ? 2048 : (g.dim == 2 ? 64 : 8);
   p->fuse_box[1] = g.dim == 1 ? 1 : (g.dim == 2 ? 16 : 8);
   p->fuse_box[2] = g.dim == 3 ? 6 : 1;
+  if (march_supported(g, dtype))
+    for (int tma = 0; tma < 2; ++tma)
+      if (g.dim == 2)
+        march2_table(g, dtype, p->sms, &p->step_table[tma]);
+      else
+        march3_table(g, dtype, p->sms, tma == 1, &p->step_table[tma]);
   p->stencil = default_stencil(p);
+  p->auto_stencil = true;
   *out = p;
   return QW_OK;
 }
@@ -350,23 +371,40 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     QW_CHECK_CUDA(cudaMemsetAsync(p->scratch, kPoisonByte, (size_t)p->g.elems * p->elem_bytes, s));
   void* cur = psi;
   void* nxt = p->scratch;
-  int64_t march[5] = {0, 0, 0, 0, 0};  // PLAIN on the square lattice and BCC boxes: launches of 1..4 steps left
   const bool marching = variant == QW_STENCIL_PLAIN && march_supported(p->g, p->dtype);
-  if (marching) march_schedule(p->g, p->dtype, nsteps, p->sms, march);
-  March1 chain{0, 0};  // PLAIN on the chain: launches left
-  if (variant == QW_STENCIL_PLAIN && p->g.dim == 1) chain = march1_schedule(p->g.nx, p->dtype, nsteps, p->sms);
-  int last = 0;  // steps of the launch before: the same kernel again may start while it drains
+  const StepTable& table = p->step_table[p->auto_stencil && aligned16(psi) ? 1 : 0];
+  int64_t march[5] = {0, 0, 0, 0, 0};  // PLAIN on the square lattice and BCC boxes: launches of 1..4 steps left
+  March1 chain{0, 0};                  // PLAIN on the chain: launches left
+  if (variant == QW_STENCIL_PLAIN) {
+    plan_run(p, nsteps, (int)(&table - p->step_table));
+    for (int t = 0; t < 5; ++t) march[t] = p->run_march[t];
+    chain = p->run_chain;
+  }
+  int last = 0;  // steps of the marching launch before: the same kernel again may start while it drains
   for (int64_t i = 0; i < nsteps;) {
     int done = 1;
     if (marching) {
       done = march[4] ? 4 : march[3] ? 3 : march[2] ? 2 : 1;
       --march[done];
-      st = p->g.dim == 2 ? launch_march2(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, done == last, s)
-                         : launch_march3(p->g, p->dtype, done, p->n, p->mass, cur, nxt, p->sms, done == last, s);
+      const int kernel = table.kernel[done];
+      if (kernel == kSiteStep)
+        st = launch_step(p->g, p->dtype, QW_STENCIL_PLAIN, p->n, p->mass, cur, nxt, s);
+      else if (kernel == kTmaStep)
+        st = launch_step_tma(p->g, p->n, p->mass, cur, nxt, p->tma_items, p->tma_nitems, p->dev_flags,
+                             p->dev_flags + 1, s);
+      else if (kernel == kTma2Step)
+        st = launch_step_tma2(p->g, p->n, p->mass, cur, nxt, p->tma2_items, p->tma2_nitems, p->dev_flags,
+                              p->dev_flags + 1, s);
+      else if (p->g.dim == 2)
+        st = launch_march2(p->g, kernel, p->n, p->mass, cur, nxt, p->sms, done == last, s);
+      else
+        st = launch_march3(p->g, p->dtype, kernel, p->n, p->mass, cur, nxt, p->sms, done == last, s);
+      last = kernel >= 0 ? done : 0;
     } else if (chain.launches > 0) {
       done = (int)((nsteps - i + chain.launches - 1) / chain.launches);
       --chain.launches;
       st = launch_march1(p->g.nx, p->dtype, chain.K, done, p->n, p->mass, cur, nxt, p->sms, last > 0, s);
+      last = done;
     } else if (variant == QW_STENCIL_TMA2 && nsteps - i >= 2) {
       st = launch_step_tma2(p->g, p->n, p->mass, cur, nxt, p->tma2_items, p->tma2_nitems, p->dev_flags,
                             p->dev_flags + 1, s);
@@ -385,7 +423,6 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     cur = nxt;
     nxt = t;
     i += done;
-    last = done;
   }
   if (cur != psi)
     QW_CHECK_CUDA(cudaMemcpyAsync(psi, cur, (size_t)p->g.elems * p->elem_bytes, cudaMemcpyDeviceToDevice, s));
@@ -399,6 +436,7 @@ qw_status qw_plan_set_stencil(qw_plan p, int variant) {
   }
   if (variant == QW_STENCIL_AUTO) {
     p->stencil = default_stencil(p);
+    p->auto_stencil = true;
     return QW_OK;
   }
   if (variant == QW_STENCIL_FUSED ? !fused_step_supported(p->g, p->dtype, p->fuse_depth, p->fuse_box)
@@ -408,6 +446,7 @@ qw_status qw_plan_set_stencil(qw_plan p, int variant) {
     return QW_EINVAL;
   }
   p->stencil = variant;
+  p->auto_stencil = false;
   return QW_OK;
 }
 
@@ -484,6 +523,7 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
                                              stencil_supported(p->g, p->dtype, v));
     if (ok) {  // the measured choice of an earlier run on this GPU model
       p->stencil = v;
+      p->auto_stencil = v == QW_STENCIL_PLAIN;
       if (v == QW_STENCIL_FUSED) {
         p->fuse_depth = dpt;
         for (int a = 0; a < 3; ++a) p->fuse_box[a] = box[a];
@@ -501,6 +541,7 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   const int saved = p->stencil, saved_depth = p->fuse_depth;
+  const bool saved_auto = p->auto_stencil;
   const int saved_box[3] = {p->fuse_box[0], p->fuse_box[1], p->fuse_box[2]};
   int best = saved, best_depth = saved_depth, best_box[3] = {saved_box[0], saved_box[1], saved_box[2]};
   double best_r = -1.0;
@@ -524,6 +565,7 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
                                 : !stencil_supported(p->g, p->dtype, c.v))
       continue;
     p->stencil = c.v;
+    p->auto_stencil = c.v == QW_STENCIL_PLAIN;
     if (c.v == QW_STENCIL_FUSED) {
       p->fuse_depth = c.depth;
       for (int a = 0; a < 3; ++a) p->fuse_box[a] = c.box[a];
@@ -554,6 +596,7 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
   cudaStreamSynchronize(s);
   cudaFree(tmp);
   p->stencil = (st == QW_OK) ? best : saved;
+  p->auto_stencil = st == QW_OK ? best == QW_STENCIL_PLAIN : saved_auto;
   if (best_rate) *best_rate = best_r;
   if (st != QW_OK) return st;
   st = check_flags(p, s);

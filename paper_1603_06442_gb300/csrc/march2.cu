@@ -71,41 +71,33 @@ qw_status launch_strips(const March2& p, const Coef32& cf, bool overlap, cudaStr
   return launch_overlapped(k, (unsigned)((items + NW - 1) / NW), 32 * NW, smem, overlap, st, p, cf);
 }
 
-const Strip2* strip2(int steps) {
-  for (const Strip2& s : kStrips)
-    if (s.t == steps) return &s;
-  return nullptr;
-}
-
 }  // namespace
 
-double march2_cost(const Geometry& g, qw_dtype dt, int steps, int sms) {
+void march2_table(const Geometry& g, qw_dtype dt, int sms, StepTable* t) {
+  for (int i = 0; i <= 4; ++i) t->kernel[i] = kNoStep;
   // one thread per site: launches and HBM at 90 G site-steps/s (complex64), or the FP64 pipe
-  if (steps == 1) return 4.0 + (double)g.sites / (dt == QW_C64 ? 90.0e3 : 7.8e3);
-  const Strip2* s = dt == QW_C64 ? strip2(steps) : nullptr;
-  if (!s) return -1.0;
-  double us;
-  geometry2(g.nx, *s, sms, &us);
-  return us;
+  t->us[1] = 4.0 + (double)g.sites / (dt == QW_C64 ? 90.0e3 : 7.8e3);
+  t->kernel[1] = kSiteStep;
+  if (dt != QW_C64) return;
+  for (int i = 0; i < (int)(sizeof(kStrips) / sizeof(Strip2)); ++i) {
+    const Strip2& s = kStrips[i];
+    geometry2(g.nx, s, sms, &t->us[s.t]);
+    t->kernel[s.t] = i;
+  }
 }
 
-qw_status launch_march2(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
-                        int sms, bool overlap, cudaStream_t st) {
-  if (steps == 1) return launch_step(g, dt, QW_STENCIL_PLAIN, n, m, in, out, st);
-  const Strip2* s = dt == QW_C64 ? strip2(steps) : nullptr;
-  if (!s) {
-    set_error("marching stencil: no kernel for %d steps", steps);
-    return QW_EINVAL;
-  }
+qw_status launch_march2(const Geometry& g, int kernel, double n, double m, const void* in, void* out, int sms,
+                        bool overlap, cudaStream_t st) {
+  const Strip2& s = kStrips[kernel];
   double us;
-  March2 p = geometry2(g.nx, *s, sms, &us);
+  March2 p = geometry2(g.nx, s, sms, &us);
   for (int q = 0; q < 4; ++q) {
     p.in[q] = static_cast<const float2*>(in) + q * g.vol;
     p.out[q] = static_cast<float2*>(out) + q * g.vol;
   }
   const Coef32 cf = make_coef32(2, n, m);
 #define X(kx, T, nw, ctas, full, own) \
-  if (s->t == T) return launch_strips<kx, T, nw, ctas>(p, cf, overlap, st);
+  if (s.t == T) return launch_strips<kx, T, nw, ctas>(p, cf, overlap, st);
   QW_STRIPS2(X)
 #undef X
   return QW_EINVAL;
@@ -116,34 +108,38 @@ bool march_supported(const Geometry& g, qw_dtype) { return g.dim >= 2 && g.vol <
 
 // The cheapest mix by the estimates; an odd number of launches ends in the scratch field and costs a
 // copy of the field.
-void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]) {
-  double cost[5];
-  for (int t = 1; t <= 4; ++t) cost[t] = g.dim == 2 ? march2_cost(g, dt, t, sms) : march3_cost(g, dt, t, sms);
-  const double copy = 3.0 + 2.0 * (double)g.elems * (dt == QW_C64 ? 8 : 16) / 6.0e6;
+void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, const StepTable& table, int64_t (&count)[5]) {
+  const double bytes = (double)g.elems * (dt == QW_C64 ? 8 : 16);
+  const double copy = 4.6 + 2.0 * bytes / (bytes < 33e6 ? 16.0e6 : 6.8e6);  // 4.6 after a kernel; L2 or HBM
   double best = -1.0;
   for (int64_t& c : count) c = 0;
   // small counts of three of the sizes, the rest in launches of the fourth
-  for (int main = 1; main <= 4; ++main) {
-    if (cost[main] < 0) continue;
+  for (int main = 1; main <= 4 && main <= nsteps; ++main) {
+    if (table.kernel[main] == kNoStep) continue;
     int64_t k[5] = {0, 0, 0, 0, 0};
     const int a = main == 1 ? 2 : 1, b = main <= 2 ? 3 : 2, c = main <= 3 ? 4 : 3;
-    const int most[5] = {0, cost[1] < 0 ? 0 : 4, cost[2] < 0 ? 0 : 4, cost[3] < 0 ? 0 : 4, cost[4] < 0 ? 0 : 4};
-    for (k[a] = 0; k[a] <= most[a]; ++k[a])
-      for (k[b] = 0; k[b] <= most[b]; ++k[b])
-        for (k[c] = 0; k[c] <= most[c]; ++k[c]) {
-          const int64_t left = nsteps - a * k[a] - b * k[b] - c * k[c];
-          if (left < 0 || left % main) continue;
+    auto most = [&](int t, int64_t left) { return table.kernel[t] == kNoStep ? 0 : std::min<int64_t>(4, left / t); };
+    const int64_t ma = most(a, nsteps);
+    for (k[a] = 0; k[a] <= ma; ++k[a]) {
+      const int64_t la = nsteps - a * k[a], mb = most(b, la);
+      for (k[b] = 0; k[b] <= mb; ++k[b]) {
+        const int64_t lb = la - b * k[b], mc = most(c, lb);
+        for (k[c] = 0; k[c] <= mc; ++k[c]) {
+          const int64_t left = lb - c * k[c];
+          if (left % main) continue;
           k[main] = left / main;
           const int64_t launches = k[1] + k[2] + k[3] + k[4];
           double total = launches % 2 ? copy : 0.0;
           for (int t = 1; t <= 4; ++t)
-            if (k[t]) total += (double)k[t] * cost[t];
+            // the first of a marching kernel's launches does not overlap the launch before it
+            if (k[t]) total += (double)k[t] * table.us[t] + (table.kernel[t] >= 0 ? kFirstMarch : 0.0);
           if (best < 0 || total < best) {
             best = total;
             for (int t = 1; t <= 4; ++t) count[t] = k[t];
           }
         }
-    k[main] = 0;
+      }
+    }
   }
 }
 

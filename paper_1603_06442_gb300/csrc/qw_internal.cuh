@@ -173,17 +173,24 @@ qw_status launch_step_tma2(const Geometry& g, double n, double m, const void* in
                            int nitems, int* err, int* next_item, cudaStream_t st);
 qw_status launch_step_tma(const Geometry& g, double n, double m, const void* in, void* out, const int4* items,
                           int nitems, int* err, int* next_item, cudaStream_t st);
+// A run of qw_step is made of launches of 1..4 steps (square lattice, BCC): for each step count the
+// estimated us of a launch and the kernel that makes it, a marching kernel's index or one of these.
+enum { kSiteStep = -1, kTmaStep = -2, kTma2Step = -3, kNoStep = -4 };
+constexpr double kFirstMarch = 2.0;  // us that a launch takes longer where it does not overlap the one before
+struct StepTable {
+  double us[5];
+  int kernel[5];
+};
 // Marching kernels (march2.cu: square lattice, march3.cu: BCC): `steps` (1..4) updates
-// out = U^steps in per launch, the steps between held in registers.  The costs are estimates in us
-// of one launch, < 0 where no kernel takes that many steps; march_schedule: how many launches of
-// 1..4 steps make nsteps.
+// out = U^steps in per launch, the steps between held in registers.  marchN_table fill the table of a
+// geometry (tma: the TMA kernels may be used); march_schedule: how many launches of 1..4 steps make nsteps.
 bool march_supported(const Geometry& g, qw_dtype dt);
-double march2_cost(const Geometry& g, qw_dtype dt, int steps, int sms);
-double march3_cost(const Geometry& g, qw_dtype dt, int steps, int sms);
-void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, int sms, int64_t (&count)[5]);
-qw_status launch_march2(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
-                        int sms, bool overlap, cudaStream_t st);
-qw_status launch_march3(const Geometry& g, qw_dtype dt, int steps, double n, double m, const void* in, void* out,
+void march2_table(const Geometry& g, qw_dtype dt, int sms, StepTable* t);
+void march3_table(const Geometry& g, qw_dtype dt, int sms, bool tma, StepTable* t);
+void march_schedule(const Geometry& g, qw_dtype dt, int64_t nsteps, const StepTable& table, int64_t (&count)[5]);
+qw_status launch_march2(const Geometry& g, int kernel, double n, double m, const void* in, void* out, int sms,
+                        bool overlap, cudaStream_t st);
+qw_status launch_march3(const Geometry& g, qw_dtype dt, int kernel, double n, double m, const void* in, void* out,
                         int sms, bool overlap, cudaStream_t st);
 // The chain (march1.cu): `launches` launches with K sites per lane make nsteps steps.
 struct March1 {
@@ -326,8 +333,15 @@ struct qw_plan_s {
   qw_dtype dtype;
   int device;
   int sms;              // multiprocessors of the device
+  qw::StepTable step_table[2];  // of the square lattice or BCC box; [1]: the TMA kernels too (BCC, AUTO, aligned fields)
+  // launches of the last run of qw_step, by step count (march) or all of one kind (chain)
+  int64_t run_steps;
+  int run_table;
+  int64_t run_march[5];
+  qw::March1 run_chain;
   size_t elem_bytes;
   int stencil;          // qw_stencil_variant in use (never AUTO after creation)
+  bool auto_stencil;    // it is AUTO's choice: single steps of PLAIN may take the TMA kernels
   int fuse_depth;       // FUSED variant: steps per launch and tile box (x, y, z cells)
   int fuse_box[3];
   void* scratch;        // one field: ping-pong partner of the caller's buffer

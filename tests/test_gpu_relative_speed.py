@@ -52,3 +52,24 @@ def test_chains_of_a_batch_keep_their_threads(qb):
     batch.sync()
     batch.close()
     assert ms < 2.5 * best_ms(lambda: qb.qw_step_static(1, N, 0.1, "c64", x, t), 2), ms
+
+
+def test_a_single_step_of_a_large_box_is_as_fast_as_the_tma_kernel(qb):
+    """1.27 of its time with the marching kernel's single step (a copy of the field included in both)."""
+    plan = qb.Plan(3, 512, 0.1, "c64")
+    x = torch.zeros(plan.elems, dtype=torch.complex64, device="cuda")
+    ms = best_ms(lambda: plan.step(x, 1), 5)
+    plan.set_stencil("tma")
+    want = best_ms(lambda: plan.step(x, 1), 5)
+    plan.close()
+    assert ms < 1.1 * want, (ms, want)
+
+
+def test_small_complex128_boxes_step_as_fast_as_a_thread_per_site(qb):
+    """1.77 of its time with the marching kernel."""
+    plan = qb.Plan(3, 48, 0.1, "c128")
+    x = torch.zeros(plan.elems, dtype=torch.complex128, device="cuda")
+    ms = best_ms(lambda: plan.step(x, 20))
+    plan.close()
+    want = best_ms(lambda: qb.qw_step_static(3, 48, 0.1, "c128", x, 20))
+    assert ms < 1.2 * want, (ms, want)
