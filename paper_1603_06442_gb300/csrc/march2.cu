@@ -26,7 +26,7 @@ struct Strip2 {
   int kx, t, nw, ctas;
   double full, own;
 };
-#define QW_STRIPS2(X) X(2, 4, 4, 2, 1.00, 0.45) X(2, 3, 4, 3, 1.25, 0.36) X(2, 2, 4, 4, 1.55, 0.27)
+#define QW_STRIPS2(X) X(2, 4, 4, 2, 1.00, 0.45) X(2, 3, 4, 3, 1.25, 0.36) X(2, 2, 4, 4, 1.66, 0.27)
 #define X(kx, t, nw, ctas, full, own) {kx, t, nw, ctas, full, own},
 const Strip2 kStrips[] = {QW_STRIPS2(X)};
 #undef X
@@ -75,8 +75,9 @@ qw_status launch_strips(const March2& p, const Coef32& cf, bool overlap, cudaStr
 
 void march2_table(const Geometry& g, qw_dtype dt, int sms, StepTable* t) {
   for (int i = 0; i <= 4; ++i) t->kernel[i] = kNoStep;
-  // one thread per site: launches and HBM at 90 G site-steps/s (complex64), or the FP64 pipe
-  t->us[1] = 4.0 + (double)g.sites / (dt == QW_C64 ? 90.0e3 : 7.8e3);
+  // one thread per site: launches and HBM at 90 G site-steps/s (complex64: N = 2998 101 us; two steps a launch
+  // 114 us, with a copy of the field where the run has no second one), or the FP64 pipe
+  t->us[1] = std::max(4.1, 2.0 + (double)g.sites / (dt == QW_C64 ? 90.0e3 : 7.8e3));
   t->kernel[1] = kSiteStep;
   if (dt != QW_C64) return;
   for (int i = 0; i < (int)(sizeof(kStrips) / sizeof(Strip2)); ++i) {
