@@ -403,7 +403,8 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
     } else if (chain.launches > 0) {
       done = (int)((nsteps - i + chain.launches - 1) / chain.launches);
       --chain.launches;
-      st = launch_march1(p->g.nx, p->dtype, chain.K, done, p->n, p->mass, cur, nxt, p->sms, last > 0, s);
+      st = chain.K == 0 ? launch_step(p->g, p->dtype, QW_STENCIL_PLAIN, p->n, p->mass, cur, nxt, s)
+                        : launch_march1(p->g.nx, p->dtype, chain.K, done, p->n, p->mass, cur, nxt, p->sms, last > 0, s);
       last = done;
     } else if (variant == QW_STENCIL_TMA2 && nsteps - i >= 2) {
       st = launch_step_tma2(p->g, p->n, p->mass, cur, nxt, p->tma2_items, p->tma2_nitems, p->dev_flags,

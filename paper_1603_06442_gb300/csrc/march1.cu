@@ -95,16 +95,23 @@ __global__ void __launch_bounds__(32 * kWarps1)
   }
 }
 
+// Few windows: a warp per CTA, so that they spread over the SMs.
+int cta_warps(int64_t windows, int sms) { return windows < (int64_t)kWarps1 * sms ? 1 : kWarps1; }
+
 // us of one launch of `steps` steps with K sites per lane.
 template <typename R> double cost1(int64_t N, int K, int steps, int sms) {
   constexpr bool f32 = sizeof(R) == 4;
   const int64_t windows = (N + 32 * K - 2 * steps - 1) / (32 * K - 2 * steps);
-  const double per_sm = (double)((windows + sms - 1) / sms);
+  // warps of the fullest SM; its CTAs come and go whole, which the FP64 pipe feels (in FP32 they hide in the waits)
+  const int warps = f32 ? 1 : cta_warps(windows, sms);
+  const int64_t ctas = (windows + warps - 1) / warps;
+  const double per_sm = (double)((ctas + sms - 1) / sms * warps);
   // clocks of a step: a warp on its own (issue and the shuffle's latency; FP64: 8 instructions a
   // site of 64 clocks each, half a lane a clock on its quarter of the SM), or all warps of an SM
-  // (FP32: 16 instructions a site on four schedulers; FP64: 8 of 16 clocks each)
+  // (FP32: 16 instructions a site on four schedulers; FP64: 8 of 16 clocks each, measured 141 with many steps a
+  // launch and 149 with one)
   const double own = f32 ? 16.0 * K + 45.0 : 512.0 * K + 60.0;
-  const double all = per_sm * K * (f32 ? 4.4 : 128.0);
+  const double all = per_sm * K * (f32 ? 4.4 : 140.0 + 9.0 / steps);
   const double compute = steps * std::max(own, all) / 1900.0;
   const double bytes = 2.0 * 2.0 * (f32 ? 8.0 : 16.0) * (double)N / 5.5e6;
   return 2.5 + std::max(compute, bytes);
@@ -115,8 +122,7 @@ qw_status launch1(const void* in, void* out, int64_t N, int steps, typename Coef
                   bool overlap, cudaStream_t st) {
   using C = typename CplxOf<R>::T;
   const int64_t windows = (N + 32 * K - 2 * steps - 1) / (32 * K - 2 * steps);
-  // few windows: a warp per CTA, so that they spread over the SMs
-  const int warps = windows < (int64_t)kWarps1 * sms ? 1 : kWarps1;
+  const int warps = cta_warps(windows, sms);
   return launch_overlapped(march1d_kernel<R, K>, (unsigned)((windows + warps - 1) / warps), 32 * warps, 0, overlap,
                            st, static_cast<const C*>(in), static_cast<C*>(out), N, steps, windows, cf);
 }
@@ -125,12 +131,19 @@ qw_status launch1(const void* in, void* out, int64_t N, int steps, typename Coef
 
 // The launches that make nsteps: sites per lane and the number of launches, whose steps differ by
 // at most one.  Long chains take the widest window (least overlap); short ones narrower windows on
-// more SMs, and as many steps a launch as pay for its start.
+// more SMs, and as many steps a launch as pay for its start.  K = 0: a launch of a thread per site for
+// every step, for complex128 chains that fill the SMs (bound by the same FP64 instructions, and none in a
+// halo: N = 20 000 003 310 us a step against 317) and single steps of the shorter ones.
 March1 march1_schedule(int64_t N, qw_dtype dt, int64_t nsteps, int sms) {
   const bool f32 = dt == QW_C64;
-  const double copy = 3.0 + 4.0 * (f32 ? 8.0 : 16.0) * (double)N / 6.0e6;
+  const double bytes = 2.0 * (f32 ? 8.0 : 16.0) * (double)N;
+  const double copy = f32 ? 3.0 + 2.0 * bytes / 6.0e6 : 4.6 + 2.0 * bytes / (bytes < 33e6 ? 16.0e6 : 6.8e6);
   March1 best{1, nsteps};
   double bc = -1.0;
+  if (!f32) {
+    bc = (double)nsteps * std::max(4.1, 3.5 + (double)N / 65.4e3) + (nsteps % 2 ? copy : 0.0);
+    best.K = 0;
+  }
   for (int K : {1, 2, 4, 8, 16}) {
     if (K == 16 && !f32) continue;
     for (int t : {1, 2, 3, 4, 6, 8, 10, 12, 14, 16, 18, 20, 24, 28, 32, 40, 48, 64, 80, 96}) {
@@ -139,8 +152,14 @@ March1 march1_schedule(int64_t N, qw_dtype dt, int64_t nsteps, int sms) {
         const int64_t k = (nsteps + t - 1) / t + odd;
         if (k > nsteps) continue;
         const int steps = (int)((nsteps + k - 1) / k);
-        const double c = (double)k * (f32 ? cost1<float>(N, K, steps, sms) : cost1<double>(N, K, steps, sms)) +
-                         (k % 2 ? copy : 0.0);
+        double c = k % 2 ? copy : 0.0;
+        if (f32) {
+          c += (double)k * cost1<float>(N, K, steps, sms);
+        } else {
+          const int64_t full = nsteps - k * (steps - 1);  // launches of `steps`; the others take one step less
+          c += kFirstMarch + (double)full * cost1<double>(N, K, steps, sms);
+          if (full < k) c += (double)(k - full) * cost1<double>(N, K, steps - 1, sms);
+        }
         if (bc < 0 || c < bc) {
           bc = c;
           best = March1{K, k};

@@ -192,7 +192,8 @@ qw_status launch_march2(const Geometry& g, int kernel, double n, double m, const
                         bool overlap, cudaStream_t st);
 qw_status launch_march3(const Geometry& g, qw_dtype dt, int kernel, double n, double m, const void* in, void* out,
                         int sms, bool overlap, cudaStream_t st);
-// The chain (march1.cu): `launches` launches with K sites per lane make nsteps steps.
+// The chain (march1.cu): `launches` launches with K sites per lane make nsteps steps (K = 0: a thread per site,
+// one step each).
 struct March1 {
   int K;
   int64_t launches;
