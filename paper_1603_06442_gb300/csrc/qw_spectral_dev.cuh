@@ -841,12 +841,6 @@ __device__ __forceinline__ void evolve_bcc_row(const AxesDev& a, int k, float4 r
   }
 }
 
-// 1 / sqrt(x) for x > 0 in FP32 with one Newton step.
-__device__ __forceinline__ float rsqrt_newton(float x) {
-  const float r = rsqrtf(x);
-  return r * fmaf(-0.5f * x * r, r, 1.5f);
-}
-
 // The coefficients of one wave vector from the four products p = sqrt((1 -+ vW)(1 +- vD)) (ae, be, af,
 // bf: a = 1 - vW, b = 1 + vW, e = 1 + vD, f = 1 - vD; every A, B, C, D of fw_apply is one of them).
 __device__ __forceinline__ void fw_row_apply(float ae, float be, float af, float bf, float ec, float es,
@@ -867,27 +861,34 @@ __device__ __forceinline__ void fw_row_apply(float ae, float be, float af, float
   v[3] = w3;
 }
 
-// fw_point for a BCC cell in complex64 from its row constants rc and x frequency k.  The half
-// spectrum q1 has the opposite n~: vW and e^{i phi} change sign, vD stays (with the 0/0 conventions of
-// fw_apply), so the square roots serve both.
-__device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, float4 rc, const Mass& ms, float scale,
+// fw_point for a BCC cell in complex64 from its row constants rc, the sum fyz of its y and z frequencies and
+// its x frequency k.  The half spectrum q1 has the opposite n~: vW and e^{i phi} change sign, vD stays (with the
+// 0/0 conventions of fw_apply), so the square roots serve both.  The coset phase is that of the exact index, as
+// coset_phase takes it (the product of the table entries carries three roundings), and e^{i phi} that of correctly
+// rounded quotients: rms error against 64 bits at N = 288, m = 0.3 2.86e-7 of the norm (3.0e-7 with the product and
+// a reciprocal square root; fw_point's 2.92e-7), m = 0.05 2.86e-7 (fw_point's 4.25e-7).
+__device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, int fyz, float4 rc, const Mass& ms, float scale,
                                            float2 (&v)[8]) {
   float cx, sx;
   tab<float>(a, 0, k, cx, sx);
   const float nx = sx * rc.x - cx * rc.y, ny = cx * rc.z + sx * rc.w, nz = cx * rc.w - sx * rc.z;
-  const float pr = rc.x - rc.y, pim = rc.w + rc.z;
-  const float ar = cx * pr - sx * pim, ai = cx * pim + sx * pr;  // a = exp(i (k1 + k2 + k3) / 2)
+  const int M = (int)a.len[0];
+  int q = k + fyz;  // below 3 M
+  q = q >= 2 * M ? q - 2 * M : q;
+  float ar, ai;
+  sincospif((float)q / (float)M, &ai, &ar);  // a = exp(i (k1 + k2 + k3) / 2)
   const float wa2 = fmaf(nx, nx, ny * ny), r2 = fmaf(nz, nz, wa2);
   constexpr float tiny2 = 1e-12f;  // (1e-6)^2, as in fw_apply
   const bool has_w = wa2 > tiny2, has_r = r2 >= tiny2;
-  const float iwa = has_w ? rsqrt_newton(wa2) : 0.f;
-  // correctly rounded: 1 -+ vW and 1 - vD must vanish where n~ lies along z or m = 0 (an error of an
-  // ulp in vW would be one of 2e-4 in its square root)
-  const float r = sqrtf(r2);
-  const float vW = has_r ? fminf(1.f, fmaxf(-1.f, -nz / r)) : 0.f;
-  const float den2 = fmaf(ms.nf * ms.nf, r2, ms.mf * ms.mf);
-  const float vD = den2 > tiny2 ? fminf(1.f, ms.nf * r / sqrtf(den2)) : 0.f;
-  const float pa = 1.f - vW, pb = 1.f + vW, pe = 1.f + vD, pf = 1.f - vD;
+  const float wa = sqrtf(wa2), ec = has_w ? -nx / wa : 1.f, es = has_w ? -ny / wa : 0.f;
+  // 1 -+ vW and 1 - vD without the difference of two numbers near 1 (an error of an ulp in vW would be one of 2e-4
+  // in its square root): (1 - |vW|) (1 + |vW|) = wa^2 / r^2, (1 - vD) (1 + vD) = m^2 / den^2
+  const float r = sqrtf(r2), az = fabsf(nz);
+  const float big = has_r ? 1.f + az / r : 1.f, small = has_r ? wa2 / (r * (r + az)) : 1.f;
+  const float pa = nz >= 0.f ? big : small, pb = nz >= 0.f ? small : big;  // 1 - vW, 1 + vW
+  const float den2 = fmaf(ms.nf * ms.nf, r2, ms.mf * ms.mf), den = sqrtf(den2), nr = ms.nf * r;
+  const bool has_d = den2 > tiny2;
+  const float pe = has_d ? 1.f + nr / den : 1.f, pf = has_d ? ms.mf * ms.mf / (den * (den + nr)) : 1.f;
   const float hs = 0.25f * scale;  // the halves of the coset mix and of the eigenvectors
   const float ae = hs * sqrtf(pa * pe), be = hs * sqrtf(pb * pe), af = hs * sqrtf(pa * pf), bf = hs * sqrtf(pb * pf);
   float2 c0[4], c1[4];
@@ -897,8 +898,8 @@ __device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, float4 rc, c
     c0[q] = make_float2(v[q].x + bx, v[q].y + by);
     c1[q] = make_float2(v[q].x - bx, v[q].y - by);
   }
-  fw_row_apply(ae, be, af, bf, has_w ? -nx * iwa : 1.f, -ny * iwa, c0);
-  fw_row_apply(be, ae, bf, af, has_w ? nx * iwa : 1.f, ny * iwa, c1);
+  fw_row_apply(ae, be, af, bf, ec, es, c0);
+  fw_row_apply(be, ae, bf, af, has_w ? -ec : 1.f, -es, c1);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const float dx = c0[q].x - c1[q].x, dy = c0[q].y - c1[q].y;
@@ -992,7 +993,14 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
     const bool ok = cc < CU && row0 + w < nrows;
     if (cc < C) cp_async_elem(&sm[cc + CP * xx], ok ? data + p * count + (row0 + w) * L + xx : data, ok);
   }
-  if (bcc_rows && tid < RW && row0 + tid < nrows) rowc[tid] = bcc_row_consts(a, row0 + tid);  // while loading
+  __shared__ int rowf[FW ? 8 : 1];  // FW: the row's fy + fz
+  if (bcc_rows && tid < RW && row0 + tid < nrows) {  // while loading
+    rowc[tid] = bcc_row_consts(a, row0 + tid);
+    if constexpr (FW) {
+      const int ny = (int)a.len[1], row = (int)(row0 + tid);
+      rowf[tid] = (int)(freq_of(row % ny, a, 1) + freq_of(row / ny, a, 2));
+    }
+  }
   cp_async_wait_all();
   __syncthreads();
   reg_fft_steps<float, false, R1, R2, CP>(sm, c, r, tw);
@@ -1007,7 +1015,7 @@ __global__ void __launch_bounds__(256, 3) fused_x_kernel(int dim, AxesDev a, int
 #pragma unroll
       for (int pp = 0; pp < 8; ++pp) v[pp] = sm[w * 8 + pp + CP * k];
       if constexpr (FW)
-        fw_bcc_row(a, k, rowc[w], ms, scale, v);
+        fw_bcc_row(a, k, rowf[w], rowc[w], ms, scale, v);
       else
         evolve_bcc_row(a, k, rowc[w], ms, nu_tab, row * L + k, ta, scale, v);
 #pragma unroll
