@@ -153,7 +153,8 @@ __device__ __forceinline__ float2 axis_factor_f(const AxisF& a, long long pos) {
 }
 
 // Rows of 256 sites (chain) or kPacketGroup rows of the box per unit; a CTA takes units in turn and
-// leaves sum |psi|^2 of what it wrote in partials (four doubles, the last three 0).
+// leaves sum |psi|^2 of what it wrote in partials (four doubles, the last three 0).  The densities of at
+// most 8 sites are summed in FP32, as the moments kernel does, and those sums in FP64.
 constexpr int kPacketGroup = 16, kPacketChain = 8;
 __global__ void __launch_bounds__(256) packet_f_kernel(Geometry g, PacketF pa, int bx, int64_t units,
                                                        float2* __restrict__ psi, double* __restrict__ partials) {
@@ -168,12 +169,14 @@ __global__ void __launch_bounds__(256) packet_f_kernel(Geometry g, PacketF pa, i
         const int64_t x = (u * kPacketChain + j) * 256 + tid;
         if (x >= g.nx) break;
         const float2 f = axis_factor_f(pa.ax[0], x);
+        float d = 0.f;
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
           const float2 v = cx_mul(f, pa.chi[q]);
           psi[q * g.vol + x] = v;
-          sum = fmaf(v.x, v.x, fmaf(v.y, v.y, sum));
+          d = fmaf(v.x, v.x, fmaf(v.y, v.y, d));
         }
+        sum += d;
       }
       acc[0] += (double)sum;
     }
@@ -196,7 +199,7 @@ __global__ void __launch_bounds__(256) packet_f_kernel(Geometry g, PacketF pa, i
       __syncthreads();
       if (ty < by && x < g.nx) {
         float sum = 0.f;
-        int cx = -1;
+        int cx = -1, sites = 0;
         float2 fx = make_float2(0.f, 0.f);
         for (int r = ty; r < kPacketGroup && row0 + r < rows; r += by) {
           const int64_t row = row0 + r;
@@ -207,11 +210,18 @@ __global__ void __launch_bounds__(256) packet_f_kernel(Geometry g, PacketF pa, i
           }
           const float2 f = cx_mul(fx, fyz[r]);
           float2* dst = psi + (int64_t)c * 3 * g.vol + row * g.nx + x;  // row counts through both cosets
+          float d = 0.f;
 #pragma unroll
           for (int q = 0; q < 4; ++q) {
             const float2 v = cx_mul(f, pa.chi[q]);
             dst[q * g.vol] = v;
-            sum = fmaf(v.x, v.x, fmaf(v.y, v.y, sum));
+            d = fmaf(v.x, v.x, fmaf(v.y, v.y, d));
+          }
+          sum += d;
+          if (++sites == 8) {
+            acc[0] += (double)sum;
+            sum = 0.f;
+            sites = 0;
           }
         }
         acc[0] += (double)sum;
