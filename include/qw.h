@@ -68,8 +68,9 @@ typedef enum { QW_C64 = 0, QW_C128 = 1 } qw_dtype;
  * launch (temporal fusion of depth 2..4, tile box and depth set by
  * qw_plan_set_fusion or the autotuner).  AUTO restores the default: PLAIN, with the
  * TMA kernels for the one- and two-step launches of large BCC boxes that they make
- * faster (complex64, a 16-byte aligned field), the fastest measured on GB300; qw_plan_autotune measures every variant (FUSED with
- * several depths and boxes) and keeps the fastest. */
+ * faster (complex64, a 16-byte aligned field), the fastest measured on GB300;
+ * qw_plan_autotune measures AUTO and every other variant (FUSED with several depths
+ * and boxes) and keeps the fastest. */
 typedef enum {
   QW_STENCIL_AUTO = 0,
   QW_STENCIL_PLAIN = 1,
@@ -138,8 +139,9 @@ qw_status qw_set_debug_poison(int on);
  * qw_batch_autotune first look in that text file for a choice measured on the
  * same GPU model for the same problem (plan: dim, N, dtype; batch: the walks'
  * (dim, N, t) and rounds_cap) and apply it without measuring; otherwise they
- * measure and append a line "<kind> <GPU model> <problem> | <values>".  The last
- * matching line wins; delete the file to re-measure.  NULL or "" turns the
+ * measure and append a line "<kind> <GPU model> kernels=<generation> <problem> |
+ * <values>".  The last matching line wins; lines of another generation of the
+ * kernels do not match; delete the file to re-measure.  NULL or "" turns the
  * cache off (the default).  Never fails (QW_OK). */
 qw_status qw_set_autotune_cache(const char* path);
 

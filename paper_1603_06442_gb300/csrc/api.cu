@@ -85,7 +85,12 @@ bool debug_poison() { return g_poison.load(std::memory_order_relaxed); }
 static std::mutex g_cache_mu;
 static std::string g_cache_path;  // empty: no autotune cache
 
-// "<kind> <GPU model> <problem>" (spaces in the model name become '_')
+// The generation of the kernels that the autotuners choose from: raised where a change of theirs can change the
+// choice, so that a choice among the kernels of before is not applied (2: marching kernels behind PLAIN and in
+// batches; a TMA2 or FUSED choice of before would hold N = 512 at half and long chains at a sixth of their rate).
+constexpr int kKernels = 2;
+
+// "<kind> <GPU model> kernels=<generation> <problem>" (spaces in the model name become '_')
 static std::string cache_key(const char* kind, const char* problem) {
   int dev = 0;
   cudaDeviceProp prop;
@@ -93,7 +98,7 @@ static std::string cache_key(const char* kind, const char* problem) {
   if (cudaGetDevice(&dev) == cudaSuccess && cudaGetDeviceProperties(&prop, dev) == cudaSuccess) name = prop.name;
   for (char& c : name)
     if (c == ' ') c = '_';
-  return std::string(kind) + " " + name + " " + problem;
+  return std::string(kind) + " " + name + " kernels=" + std::to_string(kKernels) + " " + problem;
 }
 
 bool autotune_cache_get(const char* kind, const char* problem, std::vector<double>* values) {
