@@ -158,7 +158,8 @@ qw_status qw_plan_get_fusion(qw_plan plan, int* depth, int* box);
 
 /* Autotuner of the stencil: times every variant that supports the plan (data
  * movement PLAIN / VEC / TMA, fusion depth 2 with TMA2, and FUSED with depth 2,
- * 3, 4 on three tile boxes per lattice) for 8 steps on a temporary
+ * 3, 4 on three tile boxes per lattice) for 24 steps (chains 96; fewer, 8 at
+ * least, where that is over 2e10 site-steps) on a temporary
  * field (allocated and freed here; the caller's fields are not touched) and keeps
  * the fastest; *best_rate (optional) receives its site-steps/s.  Synchronous.
  * Errors: QW_EINVAL, QW_ENOMEM, QW_ECUDA, QW_ETIMEOUT. */

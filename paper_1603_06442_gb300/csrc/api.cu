@@ -565,7 +565,10 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
       const int* b = boxes[p->g.dim - 1][k];
       cands.push_back({QW_STENCIL_FUSED, dpt, {b[0], b[1], b[2]}});
     }
-  const int64_t steps = 8;
+  // a run as users make it: PLAIN's launches depend on the step count (a chain takes 8 steps in one launch and a
+  // copy of the field), so 8 steps say little of 100; fewer only where a run would take a fifth of a second
+  const int64_t limit = p->g.dim == 1 ? 96 : 24;
+  const int64_t steps = std::max<int64_t>(8, std::min<int64_t>(limit, (int64_t)(2.0e10 / (double)p->g.sites)) / 8 * 8);
   for (const Cand& c : cands) {
     if (c.v == QW_STENCIL_FUSED ? !fused_step_supported(p->g, p->dtype, c.depth, c.box)
                                 : !stencil_supported(p->g, p->dtype, c.v))
@@ -576,7 +579,7 @@ qw_status qw_plan_autotune(qw_plan p, void* stream, double* best_rate) {
       p->fuse_depth = c.depth;
       for (int a = 0; a < 3; ++a) p->fuse_box[a] = c.box[a];
     }
-    st = qw_step(p, tmp, 2, s);  // warm-up
+    st = qw_step(p, tmp, steps, s);  // warm-up: the same kernels
     if (st != QW_OK) break;
     cudaEventRecord(e0, s);
     st = qw_step(p, tmp, steps, s);

@@ -1137,6 +1137,10 @@ qw_status qw_batch_autotune(qw_batch b, int64_t rounds_cap, void* stream, qw_bat
     if (st != QW_OK) break;
     t.tile_sites = ts;
     st = measure(t);
+    // marching walks have tiles of their own: without a chain the other sizes build the same schedule
+    if (b->kind == kMarchBatch &&
+        std::none_of(b->desc.begin(), b->desc.end(), [](const qw_walk& w) { return w.dim == 1; }))
+      break;
   }
   // stage 2: fused rounds, fusion depth and tile box per lattice (depth-1 walks keep the
   // best row tile of stage 1)
