@@ -345,7 +345,7 @@ static qw_status launch_2f(const FftPass& p, void* data, const void* src, cudaSt
   constexpr int TPL = R1 > R2 ? R1 : R2;
   const int64_t nlines = p.O * p.S;
   if constexpr (sizeof(T) == 8)
-    if (nlines <= 152 * (256 / TPL)) return launch_2f_nt<T, INV, R1, R2, 128>(p, data, src, st);
+    if (nlines <= (int64_t)sm_count() * (256 / TPL)) return launch_2f_nt<T, INV, R1, R2, 128>(p, data, src, st);
   return launch_2f_nt<T, INV, R1, R2, 256>(p, data, src, st);
 }
 

@@ -329,7 +329,7 @@ static int64_t kcount(const Geometry& g) { return g.vol; }
 // quarter of an SM for 64 clocks a warp, so a CTA of one warp per quarter, on as many SMs as there are.
 constexpr int kPointThreads = 256, kPointSmall = 128;
 static int point_threads(const Geometry& g, qw_dtype dt) {
-  return dt == QW_C128 && g.vol <= 152 * kPointThreads ? kPointSmall : kPointThreads;
+  return dt == QW_C128 && g.vol <= (int64_t)sm_count() * kPointThreads ? kPointSmall : kPointThreads;
 }
 // Rows of CTAs where they fill (an eighth idle at most) and fit the grid, else the box's positions in
 // one row: a box of 81^3 cells uses 81 of a row's 256 threads.  The positions' divisions cost a long
