@@ -242,11 +242,7 @@ def run_ours(args, rank, world, local):
         plan.set_stencil(args.stencil)
     kernel_name = {1: "march3d_kernel", 2: "step3d_c64_vec_kernel", 3: "step3d_c64_tma_kernel",
                    4: "step3d_c64_tma2_kernel"}[plan.stencil]
-    # stencil launches of a step.  The marching kernels take up to four steps each: 100 steps at N = 512 run as
-    # four launches of three steps and 22 of four; other workloads count the fewest possible.
-    stencil_launches = -(-S // {1: 4, 4: 2}.get(plan.stencil, 1))
-    if plan.stencil == 1 and (N, S) == (512, 100):
-        stencil_launches = 26
+    stencil_launches = plan.step_launches(S)  # of a step, from the library's schedule
     fused = S / stencil_launches   # steps per stencil launch, on average
     a = inputs.gaussian_packet(dim, N, (N / 2,) * 3, W["sigma"], W["k0"], [0.5, 0.5j, 0.5, -0.5j])
     host = torch.from_numpy(a.astype(np.complex64)).pin_memory()
@@ -356,8 +352,10 @@ def run_ours(args, rank, world, local):
                    "input": "Gaussian packet sigma=%g sites, k0=%s" % (W["sigma"], list(W["k0"]))},
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak,
+                     # the marching kernel's capture is of a four-step launch: no figure for a mix of launches
                      "traffic": (NCU_TRAFFIC_BYTES_PER_SITE[kernel_name] * sites
-                                 if kernel_name in NCU_TRAFFIC_BYTES_PER_SITE else None),
+                                 if kernel_name in NCU_TRAFFIC_BYTES_PER_SITE and (plan.stencil != 1 or fused == 4)
+                                 else None),
                      "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of this kernel at "
                                        "one BCC launch, scaled by sites (profiles/%s_bcc_N%d.txt)"
                                        % (kernel_name, 512 if plan.stencil == 1 else 384),
@@ -367,6 +365,8 @@ def run_ours(args, rank, world, local):
                      "kernel_hbm_GBps": fused_hbm,
                      "kernel_hbm_frac": fused_hbm / peak,
                      "avg_launch_ms": per_launch_ms,
+                     "avg_launch_note": "the run's time over its launches: an odd number of them adds one copy of the "
+                                        "field per run",
                      "site_steps_per_s_at_roofline": peak * 1e9 / (2 * field_bytes) * sites},
         "e2e": {"value": sites * S / (e2e_ms / 1e3), "unit": "site-steps/s",
                 "h2d_bytes_per_step": field_bytes, "d2h_bytes_per_step": 48, "ms_per_step": e2e_ms,
@@ -778,7 +778,8 @@ def batched_measurement(qb, dev, stream, runs=3, n_walks=256, autotune=True):
             "site_steps_per_s": rate, "algorithmic_GBps_at_64B": rate * 64 / 1e9,
             "frac_of_hbm_at_64B": rate * 64 / 1e9 / peak,
             "note": "one persistent launch; a round advances a tile by the autotuned fusion depth of its "
-                    "lattice (1: per-site update from HBM; >= 2: tile + halo in shared memory, one HBM read "
+                    "lattice (1: per-site update from HBM, or marching rounds of four and three steps in registers where the "
+                    "batch is large enough; >= 2: tile + halo in shared memory, one HBM read "
                     "and write per round); algorithmic bytes are the unfused 64 B per site-step",
             "autotuned_fusion_depth": {"1d": best["depth"][0], "2d": best["depth"][1], "bcc": best["depth"][2]},
             "autotuned_box": {"2d": best["box"][1][:2], "bcc": best["box"][2]},

@@ -173,6 +173,11 @@ qw_status qw_plan_autotune(qw_plan plan, void* stream, double* best_rate);
  * Errors: QW_EINVAL (null plan/pointer, nsteps < 0), QW_ECUDA. */
 qw_status qw_step(qw_plan plan, void* psi_dev, int64_t nsteps, void* stream);
 
+/* Kernel launches that qw_step makes of `nsteps` steps on a 16-byte aligned field
+ * with the plan's stencil variant (the copy back after an odd number of launches is
+ * not one); -1 for a null plan or nsteps < 0. */
+int64_t qw_plan_step_launches(qw_plan plan, int64_t nsteps);
+
 /* Build the spectral-path state of the plan: FFT pass plans and twiddle
  * tables, and the table of omega_k = atan2(sin omega_k, n u_k) (Sec. 3.2,
  * cos omega_k = n u_k) for every stored wave vector (one per site in 1D/2D; on

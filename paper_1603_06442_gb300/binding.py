@@ -83,6 +83,7 @@ _SIGS = {
     "qw_plan_field_elems": (ctypes.c_int64, [ctypes.c_void_p]),
     "qw_plan_sites": (ctypes.c_int64, [ctypes.c_void_p]),
     "qw_step": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]),
+    "qw_plan_step_launches": (ctypes.c_int64, [ctypes.c_void_p, ctypes.c_int64]),
     "qw_plan_set_stencil": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int]),
     "qw_plan_get_stencil": (ctypes.c_int, [ctypes.c_void_p]),
     "qw_plan_autotune": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_void_p, ctypes.POINTER(ctypes.c_double)]),
@@ -201,6 +202,10 @@ def qw_plan_sites(plan):
 
 def qw_step(plan, psi, nsteps, stream=None):
     _check(load().qw_step(plan, _ptr(psi), int(nsteps), _stream(stream)))
+
+
+def qw_plan_step_launches(plan, nsteps):
+    return load().qw_plan_step_launches(plan, int(nsteps))
 
 
 def qw_plan_set_stencil(plan, variant):
@@ -520,6 +525,10 @@ class Plan:
     def step(self, psi, nsteps, stream=None):
         self.check_field(psi)
         qw_step(self.handle, psi, nsteps, stream)
+
+    def step_launches(self, nsteps):
+        """Kernel launches that step(psi, nsteps) makes."""
+        return qw_plan_step_launches(self.handle, nsteps)
 
     def autotune(self, stream=None):
         return qw_plan_autotune(self.handle, stream)

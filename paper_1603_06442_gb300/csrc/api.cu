@@ -435,6 +435,20 @@ qw_status qw_step(qw_plan p, void* psi, int64_t nsteps, void* stream) {
   return QW_OK;
 }
 
+int64_t qw_plan_step_launches(qw_plan p, int64_t nsteps) {
+  if (!p || nsteps < 0) return -1;
+  if (nsteps == 0) return 0;
+  switch (p->stencil) {
+    case QW_STENCIL_TMA2: return nsteps / 2 + nsteps % 2;
+    case QW_STENCIL_FUSED: return (nsteps + p->fuse_depth - 1) / p->fuse_depth;
+    case QW_STENCIL_PLAIN: break;
+    default: return nsteps;
+  }
+  if (p->g.dim > 1 && !march_supported(p->g, p->dtype)) return nsteps;
+  plan_run(p, nsteps, p->auto_stencil ? 1 : 0);
+  return p->g.dim == 1 ? p->run_chain.launches : p->run_march[1] + p->run_march[2] + p->run_march[3] + p->run_march[4];
+}
+
 qw_status qw_plan_set_stencil(qw_plan p, int variant) {
   if (!p) {
     set_error("qw_plan_set_stencil: null plan");
