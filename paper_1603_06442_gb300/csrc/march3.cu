@@ -5,7 +5,7 @@
 // TMA kernel for M % 64 = 0, one thread per site and step otherwise): M = 256: 206 against 121;
 // M = 125: 166 against 68; M = 64: 90 against 36.  It is bound by issue slots and dependent
 // latencies (2 warps per scheduler at ~250 registers; IPC 0.55, FP32 pipe 40%), no longer by
-// shared memory (40% of the wavefront peak) or HBM (31%), so what a tile recomputes in its halo
+// shared memory (43% of the wavefront peak) or HBM (43% at M = 192, 48% at M = 256), so what a tile recomputes in its halo
 // costs directly: the tile and the number of steps are chosen by the estimate below.
 // complex128: bound by the FP64 pipe (2 lanes a clock and SM): 48 FP64 instructions a site-step
 // instead of 104, one step a launch (every recomputed site costs): M = 64: 7.9 against 5.1.

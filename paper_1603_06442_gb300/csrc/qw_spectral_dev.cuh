@@ -863,8 +863,8 @@ __device__ __forceinline__ void fw_row_apply(float ae, float be, float af, float
 
 // fw_point for a BCC cell in complex64 from its row constants rc, the sum fyz of its y and z frequencies and
 // its x frequency k.  The half spectrum q1 has the opposite n~: vW and e^{i phi} change sign, vD stays (with the
-// 0/0 conventions of fw_apply), so the square roots serve both.  The coset phase is that of the exact index, as
-// coset_phase takes it (the product of the table entries carries three roundings), and e^{i phi} that of correctly
+// 0/0 conventions of fw_apply), so the square roots serve both.  The coset phase is the table's entry of the exact
+// index (the product of the three axes' entries carries three roundings), and e^{i phi} that of correctly
 // rounded quotients: rms error against 64 bits at N = 288, m = 0.3 2.86e-7 of the norm (3.0e-7 with the product and
 // a reciprocal square root; fw_point's 2.92e-7), m = 0.05 2.86e-7 (fw_point's 4.25e-7).
 __device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, int fyz, float4 rc, const Mass& ms, float scale,
@@ -872,11 +872,14 @@ __device__ __forceinline__ void fw_bcc_row(const AxesDev& a, int k, int fyz, flo
   float cx, sx;
   tab<float>(a, 0, k, cx, sx);
   const float nx = sx * rc.x - cx * rc.y, ny = cx * rc.z + sx * rc.w, nz = cx * rc.w - sx * rc.z;
+  // a = exp(i (k1 + k2 + k3) / 2) = exp(i pi q / M): the table's entry of q mod M, with its sign
   const int M = (int)a.len[0];
   int q = k + fyz;  // below 3 M
   q = q >= 2 * M ? q - 2 * M : q;
   float ar, ai;
-  sincospif((float)q / (float)M, &ai, &ar);  // a = exp(i (k1 + k2 + k3) / 2)
+  tab<float>(a, 0, q >= M ? q - M : q, ar, ai);
+  ar = q >= M ? -ar : ar;
+  ai = q >= M ? -ai : ai;
   const float wa2 = fmaf(nx, nx, ny * ny), r2 = fmaf(nz, nz, wa2);
   constexpr float tiny2 = 1e-12f;  // (1e-6)^2, as in fw_apply
   const bool has_w = wa2 > tiny2, has_r = r2 >= tiny2;
