@@ -41,7 +41,7 @@ FALLBACK_HBM_GBS = 6800.0
 # at N=512, the launch it makes there.)
 NCU_TRAFFIC_BYTES_PER_SITE = {"step3d_c64_tma_kernel": (469785600 + 409331968) / 14155776,
                               "step3d_c64_tma2_kernel": (476398848 + 408239360) / 14155776,
-                              "march3d_kernel": (1431830000 + 1030636000) / 33554432}
+                              "march3d_kernel": (1428720000 + 1029544000) / 33554432}
 
 
 def parse():

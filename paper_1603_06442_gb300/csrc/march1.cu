@@ -5,8 +5,8 @@
 // FP32 operations per number of `finish`: at K = 16 a warp issues 256 FP32 operations and 4 shuffles
 // per step.  The outermost `steps` sites of a warp's window go stale, one per step and side, and are
 // not written: windows overlap by 2 steps.  Bound by the FP32 pipe: 16 operations a site-step.
-// Measured on one GB300, complex64: N = 20 000 003, 150 steps: 2.03 ms against 13.1 ms of the
-// shared-memory tiles (four steps a pass), 1.48 T site-steps/s; complex128: N = 1024, 512 steps (the
+// Measured on one GB300, complex64: N = 20 000 003, 150 steps: 1.93 ms against 13.1 ms of the
+// shared-memory tiles (four steps a pass), 1.56 T site-steps/s; complex128: N = 1024, 512 steps (the
 // FP64 pipe, half a lane a clock per quarter of an SM, and the start of a launch): 0.21 ms against
 // 2.10 ms of one launch a step (0.36 ms without overlapped launches).
 #include <cuda_runtime.h>

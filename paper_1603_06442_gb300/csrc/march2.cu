@@ -3,9 +3,9 @@
 // that makes a number of steps.
 //
 // complex64, one GB300: N = 2998, 150 steps: 5.8 ms against 15.3 ms of one thread per site and one
-// pass per step; G site-steps/s: N = 8192: 245 (four steps a pass) against 94.  It is bound by the FP32 pipe
-// and issue (IPC 0.64; 41 additions, 16 packed mass operations and 4 shuffles a site-step), then by
-// the halo of 8 in 64 columns; HBM is at 40%.  Measured slower (the kernel alone makes 263 at
+// pass per step; G site-steps/s: N = 8192: 245 (four steps a pass) against 94.  It is bound by issue and
+// latency at two warps per scheduler (0.58 a cycle at N = 2998, FP32 pipe 44%; 41 additions, 16 packed mass
+// operations and 4 shuffles a site-step), then by the halo of 8 in 64 columns; HBM is at 43%.  Measured slower (the kernel alone makes 263 at
 // N = 8192): rows handed from level to level one row late, so that the levels are independent (253),
 // and the sums in packed additions (244: fewer instructions, the same pipe).
 // One step, and complex128 (64 FP64 instructions a site-step on the FP64 pipe, where a recomputed
