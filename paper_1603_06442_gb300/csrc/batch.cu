@@ -253,8 +253,8 @@ __device__ __forceinline__ void fused_round(const BatchWalk& W, const int (&t3)[
         } else if (W.dim == 2) {
           core_2d<false>(cur + i - 1, cur + i + 1, cur + i - sy, cur + i + sy, cur + i, P, r, W.cf);
         } else {
-          core_3d<false>(cur + (1 - c) * 4 * P, sz, sy, z - 1 + c, z + c, y - 1 + c, y + c, x - 1 + c, x + c, P,
-                         cur + c * 4 * P + i, r, W.cf);
+          core_3d<false, false>(cur + (1 - c) * 4 * P, sz, sy, z - 1 + c, z + c, y - 1 + c, y + c, x - 1 + c, x + c, P,
+                                cur + c * 4 * P + i, r, W.cf);
         }
         if (last) {  // the tile's own cells: [H, H + e) maps to [s0, s0 + e), no wrap
           const int gx = s0[0] - H + x;
