@@ -678,14 +678,30 @@ __device__ __forceinline__ void fw_apply(T u, T nx, T ny, T nz, T n, T m, typena
     return;
   }
   const T tiny = sizeof(T) == 8 ? (T)1e-12 : (T)1e-6;
-  const T r = sqrt(nx * nx + ny * ny + nz * nz);
-  T vW = r < tiny ? (T)0 : -nz / r;
-  vW = vW > (T)1 ? (T)1 : (vW < (T)-1 ? (T)-1 : vW);
-  const T wa = sqrt(nx * nx + ny * ny);
+  const T wa2 = nx * nx + ny * ny;
+  const T r = sqrt(wa2 + nz * nz);
+  const T wa = sqrt(wa2);
   const T ec = wa > tiny ? -nx / wa : (T)1, es = wa > tiny ? -ny / wa : (T)0;
   const T den = sqrt(m * m + n * n * r * r);
-  T vD = den > tiny ? n * r / den : (T)0;
-  vD = vD > (T)1 ? (T)1 : (vD < (T)-1 ? (T)-1 : vD);
+  T pa, pb, pe, pf;  // 1 - vW, 1 + vW, 1 + vD, 1 - vD
+  if (sizeof(T) == 8) {
+    T vW = r < tiny ? (T)0 : -nz / r;
+    vW = vW > (T)1 ? (T)1 : (vW < (T)-1 ? (T)-1 : vW);
+    T vD = den > tiny ? n * r / den : (T)0;
+    vD = vD > (T)1 ? (T)1 : (vD < (T)-1 ? (T)-1 : vD);
+    pa = (T)1 - vW;
+    pb = (T)1 + vW;
+    pe = (T)1 + vD;
+    pf = (T)1 - vD;
+  } else {
+    // without the difference of two numbers near 1 (see fw_bcc_row): random fields on the square lattice, N = 128,
+    // m = 0.05: rms error 2.04e-7 of the norm (3.68e-7 with it)
+    const T az = fabs(nz), big = r < tiny ? (T)1 : (T)1 + az / r, small = r < tiny ? (T)1 : wa2 / (r * (r + az));
+    pa = nz >= (T)0 ? big : small;
+    pb = nz >= (T)0 ? small : big;
+    pe = den > tiny ? (T)1 + n * r / den : (T)1;
+    pf = den > tiny ? m * m / (den * (den + n * r)) : (T)1;
+  }
   // e^{-i phi} v1, e^{-i phi} v3
   V t1, t3;
   t1.x = ec * v[1].x + es * v[1].y;
@@ -696,10 +712,9 @@ __device__ __forceinline__ void fw_apply(T u, T nx, T ny, T nz, T n, T m, typena
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const T sg = q < 2 ? (T)1 : (T)-1, pp = (q & 1) ? (T)-1 : (T)1;
-    const T A = (T)0.5 * sqrt(((T)1 - pp * vW) * ((T)1 + sg * pp * vD));
-    const T B = (T)0.5 * sqrt(((T)1 + pp * vW) * ((T)1 + sg * pp * vD));
-    const T C = (T)0.5 * sqrt(((T)1 - pp * vW) * ((T)1 - sg * pp * vD));
-    const T D = (T)0.5 * sqrt(((T)1 + pp * vW) * ((T)1 - sg * pp * vD));
+    const T wm = (q & 1) ? pb : pa, wp = (q & 1) ? pa : pb;            // 1 -+ p vW
+    const T dp = (q < 2) == !(q & 1) ? pe : pf, dm = (q < 2) == !(q & 1) ? pf : pe;  // 1 +- s p vD
+    const T A = (T)0.5 * sqrt(wm * dp), B = (T)0.5 * sqrt(wp * dp), C = (T)0.5 * sqrt(wm * dm), D = (T)0.5 * sqrt(wp * dm);
     w[q].x = A * v[0].x - pp * B * t1.x - sg * C * v[2].x + sg * pp * D * t3.x;
     w[q].y = A * v[0].y - pp * B * t1.y - sg * C * v[2].y + sg * pp * D * t3.y;
   }
